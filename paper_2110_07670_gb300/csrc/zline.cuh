@@ -2,13 +2,12 @@
 // compile-time N^3 boxes: forward FFT along z, times the Coulomb kernel
 // 4 pi / |G|^2 / N (G = 0 dropped), inverse FFT along z.
 //
-// Geometry: every z line (pencil) belongs to two lanes of one warp (lanes l
-// and l + 16), which split its butterflies, so stages need only __syncwarp and
-// no block-wide barrier exists.  A warp owns G <= 16 consecutive pencils of
-// the plane (G consecutive complex values per z row, 8 G bytes, one bulk copy
-// each), so at every step each half-warp touches G adjacent shared-memory
-// words (no bank conflicts) and G adjacent global words (full sectors).
-// Blocks are one warp.
+// Two forms: the pass's own kernel zline_coulomb (below, pencils in pairs,
+// packed arithmetic), and pencils_compute, the persistent pipeline's
+// (pipeline.cuh), where every z line belongs to two lanes of one warp (lanes l
+// and l + 16) and a warp owns G <= 16 consecutive pencils of the plane.  Both
+// split a line's butterflies over lanes, so stages need only __syncwarp and no
+// block-wide barrier exists, and touch whole 128-byte runs at every step.
 //
 // Per pencil the stages are: forward stages 0 .. S-2 in shared memory; the
 // last forward stage, the Coulomb factors and the first inverse stage fused
@@ -114,38 +113,114 @@ __device__ __forceinline__ void pencils_compute(cx<float>* buf, const cx<float>*
     if (on) pencil_last<PL::radix(0), N, G>(col, tw, out, h);
 }
 
-template <int N, int G, int F0>
+// ---------------------------------------------------------------- the pass
+// Packed form (f2): pencils p and p + 1, neighbours in the plane's layout, run
+// through every butterfly together, one packed instruction doing the work of
+// two.  A warp owns 8 pencil pairs (128 bytes of every z row, copied by 16-byte
+// cp.async; four lanes share a pair's butterflies), a block is one warp.  A
+// pair's 16 bytes {re0, im0, re1, im1} become {re0, re1}, {im0, im1} in the
+// first stage's registers and turn back in the last's.
+// Bound: DRAM (0.85 GB per 64 transforms of 96^3 at 5.6 TB/s) with the shared
+// memory pipe at 68%.  Measured per 64 / 38 / 16 transforms of 96^3 / 120^3 /
+// 160^3: 153 / 191 / 233 us, where single pencils on two lanes each, fetched by
+// one 128-byte bulk copy per z row (some 8 instructions each: a lane's copies
+// are issued one by one), took 179 / 266 / 316.  Fully unrolled rounds (more
+// registers, more code) and persistent warps that fetch the next group behind
+// the last stage are slower (96^3 165 and 154 us).
+
+constexpr int kPairsPerWarp = 8;
+
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(smem_dst)), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+}
+__device__ __forceinline__ f2 ldg2(const float* p) {
+    f2 r;
+    r.v = __ldg(reinterpret_cast<const unsigned long long*>(p));
+    return r;
+}
+// two neighbouring complex values <-> their real and imaginary parts paired
+__device__ __forceinline__ cx<f2> swap_mid(cx<f2> a) {
+    return mk(mk_f2(lo(a.re), lo(a.im)), mk_f2(hi(a.re), hi(a.im)));
+}
+
+template <int N, int F0>
 __global__ void __launch_bounds__(32) zline_coulomb(PassArgs a) {
     using PL = CPlan<N, F0>;
-    static_assert(PL::stages >= 2, "the fused middle needs two stages or more");
-    static_assert(G % 2 == 0 && G <= 16 && (N * N) % G == 0, "pencil group");
-    constexpr long long NN = (long long)N * N;
+    using c2 = cx<f2>;
+    static_assert(PL::stages == 2 && N % 2 == 0, "two stages, pencils in pairs");
+    constexpr int U = kPairsPerWarp, L = 32 / U;
+    constexpr int R0 = PL::radix(0), R1 = PL::radix(1), M0 = N / R0, B1 = N / R1;
+    constexpr long long HU = (long long)N * N / 2;  // pencil pairs of the box
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t bar;
-    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);  // [N][G]
-    cx<float>* tw = buf + N * G;                               // [N]
-    const int lane = threadIdx.x;
-    const long long p0 = (long long)blockIdx.x * G;
+    c2* buf = reinterpret_cast<c2*>(smem_raw);                  // [N][U]
+    cx<float>* tw = reinterpret_cast<cx<float>*>(buf + N * U);  // [N]
+    const int lane = threadIdx.x, l = lane % U, h = lane / U;
+    const long long p = (long long)blockIdx.x * U + l;
     const int t = blockIdx.y;
-    const cx<float>* src = reinterpret_cast<const cx<float>*>(a.src) + t * a.src_tstride + p0;
-
-    if (lane == 0) {
-        mbar_init(&bar, 1);
-        fence_mbar_init();
-        mbar_arrive_expect_tx(&bar, (uint32_t)(N * G * sizeof(cx<float>)));
-    }
-    __syncwarp();
-    for (int z = lane; z < N; z += 32) bulk_load(buf + z * G, src + z * NN, (uint32_t)(G * sizeof(cx<float>)), &bar);
+    const bool on = HU % U == 0 || p < HU;  // lanes past the last pair only keep the barriers
+    const c2* src = reinterpret_cast<const c2*>(reinterpret_cast<const cx<float>*>(a.src) + t * a.src_tstride) + p;
+    if (on)
+#pragma unroll 4
+        for (int z = h; z < N; z += L) cp_async16(buf + z * U + l, src + z * HU);
     for (int j = lane; j < N; j += 32) tw[j] = reinterpret_cast<const cx<float>*>(a.twz)[j];
+    cp_async_wait();
     __syncwarp();
-    if (!mbar_wait_bounded(&bar, 0, a.err, 1)) {
-        // copies still in flight land in this block's shared memory: give them
-        // a second bounded wait before the block leaves
-        mbar_wait_bounded(&bar, 0, nullptr, 0);
-        return;
+    c2* col = buf + l;
+    if (on) {
+#pragma unroll 1
+        for (int j = h; j < M0; j += L) {
+            c2 u[R0];
+#pragma unroll
+            for (int k = 0; k < R0; ++k) u[k] = swap_mid(col[(j + k * M0) * U]);
+            Dft<R0, -1, f2>::run(u);
+#pragma unroll
+            for (int s = 1; s < R0; ++s) u[s] = cmul(u[s], tw[s * j]);
+#pragma unroll
+            for (int s = 0; s < R0; ++s) col[(j + s * M0) * U] = u[s];
+        }
     }
-    pencils_compute<N, G, F0>(buf, tw, reinterpret_cast<const float*>(a.kern) + p0,
-                          reinterpret_cast<cx<float>*>(a.dst) + t * a.dst_tstride + p0, lane);
+    __syncwarp();
+    if (on) {
+        // last forward stage, the Coulomb factors and the first inverse stage
+        // act on the same butterflies
+        const float* kern = reinterpret_cast<const float*>(a.kern) + 2 * p;
+#pragma unroll 1
+        for (int b = h; b < B1; b += L) {
+            f2 k[R1];
+            c2 u[R1];
+#pragma unroll
+            for (int q = 0; q < R1; ++q) k[q] = ldg2(kern + (b * R1 + q) * (2 * HU));
+#pragma unroll
+            for (int q = 0; q < R1; ++q) u[q] = col[(b * R1 + q) * U];
+            Dft<R1, -1, f2>::run(u);
+#pragma unroll
+            for (int q = 0; q < R1; ++q) u[q] = scale(u[q], k[q]);
+            Dft<R1, +1, f2>::run(u);
+#pragma unroll
+            for (int q = 0; q < R1; ++q) col[(b * R1 + q) * U] = u[q];
+        }
+    }
+    __syncwarp();
+    if (on) {
+        c2* out = reinterpret_cast<c2*>(reinterpret_cast<cx<float>*>(a.dst) + t * a.dst_tstride) + p;
+#pragma unroll 1
+        for (int j = h; j < M0; j += L) {
+            c2 u[R0];
+            u[0] = col[j * U];
+#pragma unroll
+            for (int q = 1; q < R0; ++q) {
+                cx<float> w = tw[q * j];
+                w.im = -w.im;
+                u[q] = cmul(col[(j + q * M0) * U], w);
+            }
+            Dft<R0, +1, f2>::run(u);
+#pragma unroll
+            for (int s = 0; s < R0; ++s) out[(j + s * M0) * HU] = swap_mid(u[s]);
+        }
+    }
 }
 
 }  // namespace zline_detail
@@ -153,16 +228,16 @@ __global__ void __launch_bounds__(32) zline_coulomb(PassArgs a) {
 // F0: the first radix of the z axis (0: make_axis_plan's choice)
 template <int N, int F0 = 0>
 cudaError_t zline_launch(const PassArgs& a, int batch, cudaStream_t st) {
-    constexpr int G = zline_group(N);
-    auto k = zline_detail::zline_coulomb<N, G, F0>;
+    constexpr int U = zline_detail::kPairsPerWarp;
+    auto k = zline_detail::zline_coulomb<N, F0>;
     static bool carveout = [&] {
         cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaGetLastError();
         return true;
     }();
     (void)carveout;
-    const size_t smem = (size_t)(N * G + N) * sizeof(cx<float>);
-    dim3 grid((unsigned)(N * N / G), (unsigned)batch);
+    const size_t smem = (size_t)N * U * sizeof(cx<f2>) + N * sizeof(cx<float>);
+    dim3 grid((unsigned)((N * N / 2 + U - 1) / U), (unsigned)batch);
     k<<<grid, 32, smem, st>>>(a);
     return cudaGetLastError();
 }
