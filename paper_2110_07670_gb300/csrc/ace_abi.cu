@@ -333,6 +333,15 @@ int setup_shapes(ace_plan* P) {
         const int ty = largest_divisor_at_most(n1, std::max(1, target / (n0 * tx)));
         P->s_z = mk_shape(n0, ty, tx, 4);
     }
+    // single precision: the runtime-size kernels take every box they can hold
+    // (measured against the tile passes: see generic.cuh)
+    if (sizeof(R) == 4 && generic_supported(n0, n1, n2, (size_t)smax - 2048)) {
+        P->gen = P->fused_xy = true;
+        P->s_xy = mk_shape(1, n1, n2, 3);
+        P->s_xy.gen = P->s_z.gen = 1;
+        P->ntiles_last = P->ntiles_xy = n0;
+        return ACE_OK;
+    }
     for (const PassShape* s : {&P->s_xy, &P->s_x, &P->s_y, &P->s_z}) {
         if (s == &P->s_xy && !P->fused_xy) continue;
         if (s->smem > (size_t)smax) return fail(ACE_ERR_GRID_TOO_SMALL, "grid axis too long for one thread block tile");
@@ -373,6 +382,15 @@ PassArgs base_args(const ace_plan* P) {
         ++P->launches;                                                                                        \
         if (e_ != cudaSuccess) return fail(ACE_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e_)); \
     } while (0)
+
+// The real-space functions of run_to_real are psi(r) times this number: the
+// scale Omega^-1/2 rounded to the plan's precision, over itself.  A coherent
+// error of up to 6e-8 per function in single precision; the factors applied to
+// products of functions afterwards (in double) divide it out again.
+template <typename R>
+double phi_gain(const ace_plan* P) {
+    return (double)(R)(1.0 / std::sqrt(P->omega)) * std::sqrt(P->omega);
+}
 
 // psi (half sphere) -> real-space functions out[a] (quads (a, a, c, c)).
 template <typename R>
@@ -763,10 +781,12 @@ int pairs_enqueue(ace_plan* P, const void* psi_G, int n_occ, double alpha, const
     ACE_TRY(grow(&P->d_epart, &P->epart_cap, (size_t)std::max(n_pair_t, 1) * P->ntiles_last * 2));
     ACE_TRY(run_pairs<R>(P, phi, phi, acc, acc, 1, d_pq, n_pair_t, P->d_epart, st));
     mark(P, PH_ENERGY, st);
-    ACE_CKL(launch_energy_reduce(P->d_epart, d_pq, n_pair_t, P->ntiles_last, -alpha * P->omega / (double)P->N,
-                                 P->d_E, st));
+    // the pair energies carry four functions, the accumulators three
+    const double g = phi_gain<R>(P), g3 = g * g * g;
+    ACE_CKL(launch_energy_reduce(P->d_epart, d_pq, n_pair_t, P->ntiles_last,
+                                 -alpha * P->omega / (double)P->N / (g3 * g), P->d_E, st));
     cx<R>* WG = (cx<R>*)WG_out;
-    ACE_TRY(run_to_recip<R>(P, acc, d_oq, n_orb_t, -alpha * std::sqrt(P->omega) / (double)P->N, WG, st));
+    ACE_TRY(run_to_recip<R>(P, acc, d_oq, n_orb_t, -alpha * std::sqrt(P->omega) / (double)P->N / g3, WG, st));
     ACE_CK(cudaMemcpyAsync(&P->h_res->E, P->d_E, sizeof(double), cudaMemcpyDeviceToHost, st));
     return ACE_OK;
 }
@@ -877,8 +897,9 @@ int hfx_impl(ace_plan* P, const void* psi_occ, int n_occ, double alpha, const vo
     ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi, P->d_quads + no, nt, (R*)tphi, st));
     ACE_CK(cudaMemsetAsync(P->d_tacc, 0, (size_t)T * P->N * sizeof(R), st));
     ACE_TRY(run_pairs<R>(P, (const R*)tphi, phi, (R*)P->d_tacc, nullptr, 0, P->d_quads + no + nt, np, nullptr, st));
-    ACE_TRY(run_to_recip<R>(P, (const R*)P->d_tacc, P->d_quads + no, nt, -alpha * std::sqrt(P->omega) / (double)P->N,
-                            (cx<R>*)out, st));
+    const double g = phi_gain<R>(P);
+    ACE_TRY(run_to_recip<R>(P, (const R*)P->d_tacc, P->d_quads + no, nt,
+                            -alpha * std::sqrt(P->omega) / (double)P->N / (g * g * g), (cx<R>*)out, st));
     mark(P, PH_IDLE, st);
     ACE_CK(cudaGetLastError());
     return ACE_OK;
@@ -898,7 +919,8 @@ int overlap_impl(ace_plan* P, const void* psi_G, int n, double rho_cut, int32_t*
     R* phi = (R*)P->d_phi;
     ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi_G, P->d_quads, (int)oq.size(), phi, st));
     const long long K = P->N;
-    const double scale = P->omega / (double)P->N;
+    const double g = phi_gain<R>(P);
+    const double scale = P->omega / (double)P->N / (g * g);
     mark(P, PH_GRAM, st);
     bool done = false;
     if constexpr (sizeof(R) == 4) {

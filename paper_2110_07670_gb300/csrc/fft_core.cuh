@@ -212,7 +212,10 @@ struct Dft<4, SGN, R> {
 template <int SGN, typename R>
 struct Dft<5, SGN, R> {
     // c1 = cos(2pi/5), c2 = cos(4pi/5), s1 = sin(2pi/5), s2 = sin(4pi/5);
-    // s1 b1 + s2 b2 = s1 (b1 + (s2/s1) b2), s2 b1 - s1 b2 = s2 (b1 - (s1/s2) b2)
+    // s1 b1 + s2 b2 = s2 (b2 + (s1/s2) b1), s2 b1 - s1 b2 = s2 (b1 - (s1/s2) b2):
+    // in single precision s2 and s2 (s1/s2) = s1 are off by 1.4e-8 and 0.4e-8
+    // (with s1 taken out, s1 (s2/s1) = s2 would be off by 5.1e-8, a gain error
+    // that adds up over the axes)
     static ACE_HD void run(cx<R>* v) {
         const double c1 = 0.30901699437494742410, c2 = -0.80901699437494742410;
         const double s1 = 0.95105651629515357212, s2 = 0.58778525229247312917;
@@ -221,11 +224,11 @@ struct Dft<5, SGN, R> {
         cx<R> x0 = v[0];
         cx<R> p1 = madd(madd(x0, R(c1), a1), R(c2), a2);
         cx<R> p2 = madd(madd(x0, R(c2), a1), R(c1), a2);
-        cx<R> q1 = madd(b1, R(s2 / s1), b2);
+        cx<R> q1 = madd(b2, R(s1 / s2), b1);
         cx<R> q2 = madd(b1, R(-s1 / s2), b2);
         v[0] = (x0 + a1) + a2;
-        v[1] = madd_i<SGN>(p1, s1, q1);
-        v[4] = madd_i<-SGN>(p1, s1, q1);
+        v[1] = madd_i<SGN>(p1, s2, q1);
+        v[4] = madd_i<-SGN>(p1, s2, q1);
         v[2] = madd_i<SGN>(p2, s2, q2);
         v[3] = madd_i<-SGN>(p2, s2, q2);
     }
