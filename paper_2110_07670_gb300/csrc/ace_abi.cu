@@ -109,6 +109,7 @@ struct ace_plan {
     bool cube_kernels = true;  // compile-time kernels for supported N^3 boxes
     bool tensor_gram = false;  // Gram products on tcgen05 tensor cores (single precision)
     int lookahead = 1;         // L2 look-ahead of the pair passes, in transforms (env ACE_LOOKAHEAD)
+    bool gen = false;          // runtime-size plane / pencil kernels (generic.cuh), Coulomb factors from d_kern
     bool zline = false;        // per-pencil Coulomb pass (zline.cuh) with the kernel table d_kern
     float* d_kern = nullptr;   // 4 pi / |G|^2 / N in the tile passes' spectrum layout (zline only)
     float* d_kern_t = nullptr; // the same for transposed planes (n % 8 == 0 cubes)
@@ -1422,12 +1423,13 @@ int pair_tables(ace_plan* P, int r0) {
     }
     P->pair_r0 = r0;
     const bool swz = P->s_xy.cube && cube_swizzle(P->n[2]);
-    const bool inline_tab = !P->zline && (P->coul_rc > 0 || P->coul_g0 || sizeof(R) == 8);
-    if (!P->zline && !inline_tab) return ACE_OK;
+    const bool tab = P->zline || P->gen;
+    const bool inline_tab = !tab && (P->coul_rc > 0 || P->coul_g0 || sizeof(R) == 8);
+    if (!tab && !inline_tab) return ACE_OK;
     const int n0 = P->n[0], n1 = P->n[1], n2 = P->n[2];
     const bool with_t = P->zline && tplane_supported(n0);
     const bool swz_i = P->s_z.cube && cube_swizzle(n2);  // x slots of the tile passes' Coulomb stage
-    std::vector<float> kern(P->zline ? (size_t)P->N : 0), kern_t(with_t ? (size_t)P->N : 0);
+    std::vector<float> kern(tab ? (size_t)P->N : 0), kern_t(with_t ? (size_t)P->N : 0);
     std::vector<R> kern_r(inline_tab ? (size_t)P->N : 0);
     auto fold = [](int k, int n) { return k < n - n / 2 ? k : k - n; };
     auto g2_at = [&](int z, int y, int xp) {
@@ -1451,7 +1453,7 @@ int pair_tables(ace_plan* P, int r0) {
         for (int y = 0; y < n1; ++y)
             for (int xs = 0; xs < n2; ++xs) {
                 const size_t e = ((size_t)z * n1 + y) * n2 + xs;
-                if (P->zline) kern[e] = (float)k(g2_at(z, y, swz ? plane_swizzle(xs, y, n2) : xs));
+                if (tab) kern[e] = (float)k(g2_at(z, y, swz ? plane_swizzle(xs, y, n2) : xs));
                 if (with_t) kern_t[((size_t)z * n2 + xs) * n1 + y] = (float)k(g2_at(z, y, xs));  // plane [x][y]
                 if (inline_tab) kern_r[e] = (R)k(g2_at(z, y, swz_i ? plane_swizzle(xs, y, n2) : xs));
             }
@@ -1459,7 +1461,7 @@ int pair_tables(ace_plan* P, int r0) {
         if (!P->d_kern_t) ACE_TRY(dalloc((void**)&P->d_kern_t, kern_t.size() * sizeof(float)));
         ACE_CK(cudaMemcpy(P->d_kern_t, kern_t.data(), kern_t.size() * sizeof(float), cudaMemcpyHostToDevice));
     }
-    if (P->zline) {
+    if (tab) {
         if (!P->d_kern) ACE_TRY(dalloc((void**)&P->d_kern, kern.size() * sizeof(float)));
         ACE_CK(cudaMemcpy(P->d_kern, kern.data(), kern.size() * sizeof(float), cudaMemcpyHostToDevice));
     }

@@ -71,6 +71,7 @@ struct PassArgs {
 struct PassShape {
     int tz, ty, tx, axes, threads, bulk, vec;
     int cube;  // 1: use the compile-time kernel of this N^3 box (single precision)
+    int gen;   // 1: use the runtime-size plane / pencil kernels (single precision)
     size_t smem;
 };
 
@@ -187,6 +188,15 @@ inline bool stream_capturing(cudaStream_t st) {
 // compile-time cube passes (cube_*.cu), single precision
 cudaError_t cube_pass_launch(int n, const PassArgs& a, const PassShape& s, int pro, int epi, int mid, int sgn,
                              int batch, cudaStream_t st);
+
+// Single-precision passes on runtime-size boxes (generic.cuh), for boxes whose
+// plane and pencil group fit a block's shared memory (every extent >= 2): plane
+// passes (PRO_PAIR / PRO_PACK2 with EPI_STORE; EPI_ACCUM / EPI_SPLIT), pencil
+// passes (mode -1 forward z, +1 inverse z, 0 forward z, times PassArgs::kern,
+// inverse z).
+bool generic_supported(int n0, int n1, int n2, size_t smem_limit);
+cudaError_t generic_plane_launch(const PassArgs& a, int pro, int epi, int batch, cudaStream_t st);
+cudaError_t generic_pencil_launch(const PassArgs& a, int mode, int batch, cudaStream_t st);
 
 // Launch one pass over `batch` transforms (gridDim.y) of the box.
 template <typename R>

@@ -21,6 +21,11 @@ cudaError_t launch_pass(const PassArgs& a0, const PassShape& s, int pro, int epi
         if (sizeof(R) != 4 || a.n0 != a.n1 || a.n1 != a.n2) return cudaErrorInvalidValue;
         return cube_pass_launch(a.n0, a, s, pro, epi, mid, sgn, batch, st);
     }
+    if (s.gen) {
+        if (sizeof(R) != 4) return cudaErrorInvalidValue;
+        if (s.axes == 4) return generic_pencil_launch(a, mid == MID_COULOMB ? 0 : sgn, batch, st);
+        return generic_plane_launch(a, pro, epi, batch, st);
+    }
     return pass_detail::dispatch<pass_detail::DynShape, R>(a, s, pro, epi, mid, sgn, batch, st);
 }
 
