@@ -20,9 +20,9 @@
 //
 // Bound: instruction issue (runtime strides, about 1.6 times the compile-time
 // kernels' instructions per element).  Against the runtime-size tile passes these
-// replace, per 32 transforms of 72^3: forward planes 92 vs 127 us, pencils 50 vs
-// 347, inverse planes 96 vs 150; 64 orbitals there 7.15 vs 19.9 ms per build, 27
-// orbitals on 40 x 48 x 45 0.57 vs 1.26 ms.
+// replace, per 32 transforms of 72^3: forward planes 62 vs 127 us, pencils 48 vs
+// 347, inverse planes 93 vs 150; 64 orbitals there 6.4 vs 19.8 ms per build, 27
+// orbitals on 40 x 48 x 45 0.58 vs 1.28 ms.
 #pragma once
 
 #include "internal.h"

@@ -53,8 +53,7 @@ constexpr uint32_t TMEM_COLS = 512;  // two sets of (hi.hi, small products) x 12
 struct __align__(1024) WsSmem {
     float a_hi[NB][128 * TK];
     float a_lo[NB][128 * TK];
-    float b_hi[NB][128 * TK];
-    float b_lo[NB][128 * TK];
+    float b[NB][2][128 * TK];  // hi, lo: 256 consecutive operand rows
     uint64_t full[NB];   // producers -> MMA: buffer written (NPROD arrivals)
     uint64_t empty[NB];  // MMA -> producers: buffer read (tcgen05.commit)
     uint64_t tfull[2];   // MMA -> drain: turn complete in set (tcgen05.commit)
@@ -95,17 +94,21 @@ __device__ __forceinline__ void ws_init(WsSmem& sm, int full_count) {
 // up at once when another role has aborted.  Returns false on either.
 __device__ __forceinline__ bool ws_wait(WsSmem& sm, uint64_t* bar, long long use, int* err) {
     const uint32_t parity = (uint32_t)(use & 1);
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    while (!mbar_try_wait(bar, parity)) {
+    // the clock and the abort flag are looked at once in 32 polls: most waits end
+    // within a few, and reading the clock delays the poll that would see it
+    uint64_t t0 = 0;
+    for (uint32_t i = 0;; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((i & 31) != 31) continue;
         if (*reinterpret_cast<volatile int*>(&sm.abort)) return false;
-        if (global_ns() - t0 > 2000000000ull) {
+        const uint64_t now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 2000000000ull) {
             if (err) atomicExch(err, 2);
             *reinterpret_cast<volatile int*>(&sm.abort) = 1;
             return false;
         }
     }
-    return true;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -120,23 +123,22 @@ __device__ __forceinline__ void ws_produced(uint64_t* bar) {
     if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
 
-// The 12 MMAs of one stage (4 K steps x hi.hi, hi.lo, lo.hi) from buffer buf
-// into accumulator set `set`.
+// The 8 MMAs of one stage (4 K steps) from buffer buf into accumulator set
+// `set`: hi.[hi | lo] with both halves of B as one operand of 256 rows (columns
+// 0-127 hi.hi, 128-255 the small products), then lo.hi onto the small products.
+// (Three N = 128 products took 118 cycles each whatever the operands.)
 __device__ __forceinline__ void ws_mma(WsSmem& sm, int buf, uint32_t tmem, int set, bool first) {
-    constexpr uint32_t IDESC = umma::idesc_tf32(128, 128);
+    constexpr uint32_t IDESC = umma::idesc_tf32(128, 128), IDESC2 = umma::idesc_tf32(128, 256);
     const unsigned char* ah = reinterpret_cast<const unsigned char*>(sm.a_hi[buf]);
     const unsigned char* al = reinterpret_cast<const unsigned char*>(sm.a_lo[buf]);
-    const unsigned char* bh = reinterpret_cast<const unsigned char*>(sm.b_hi[buf]);
-    const unsigned char* bl = reinterpret_cast<const unsigned char*>(sm.b_lo[buf]);
+    const unsigned char* bb = reinterpret_cast<const unsigned char*>(sm.b[buf][0]);
     const uint32_t d = tmem + (uint32_t)set * 256;
 #pragma unroll
     for (int kk = 0; kk < TK / 8; ++kk) {
         const uint64_t dah = umma::desc_sw128(ah + kk * 32), dal = umma::desc_sw128(al + kk * 32);
-        const uint64_t dbh = umma::desc_sw128(bh + kk * 32), dbl = umma::desc_sw128(bl + kk * 32);
-        const uint32_t acc = (!first || kk > 0) ? 1u : 0u;
-        umma::mma_tf32(d + 128, dal, dbh, IDESC, acc);
-        umma::mma_tf32(d + 128, dah, dbl, IDESC, 1u);
-        umma::mma_tf32(d, dah, dbh, IDESC, acc);
+        const uint64_t db = umma::desc_sw128(bb + kk * 32);
+        umma::mma_tf32(d, dah, db, IDESC2, (!first || kk > 0) ? 1u : 0u);
+        umma::mma_tf32(d + 128, dal, db, IDESC, 1u);
     }
 }
 
@@ -213,8 +215,8 @@ __global__ void __launch_bounds__(NTHR, 1)
             if (s >= NB && !ws_wait(sm, &sm.empty[b], s / NB - 1, err)) return false;
             unsigned char* ah = reinterpret_cast<unsigned char*>(sm.a_hi[b]) + off;
             unsigned char* al = reinterpret_cast<unsigned char*>(sm.a_lo[b]) + off;
-            unsigned char* bh = reinterpret_cast<unsigned char*>(sm.b_hi[b]) + off;
-            unsigned char* bl = reinterpret_cast<unsigned char*>(sm.b_lo[b]) + off;
+            unsigned char* bh = reinterpret_cast<unsigned char*>(sm.b[b][0]) + off;
+            unsigned char* bl = reinterpret_cast<unsigned char*>(sm.b[b][1]) + off;
 #pragma unroll
             for (int u = 0; u < 16; ++u) {
                 uint32_t hx, lx, hy, ly;
@@ -273,9 +275,17 @@ __global__ void __launch_bounds__(NTHR, 1)
             const int jb = j0 + ((warp - WARP_DRAIN0) >> 2) * 64;
             if (i < m) {
                 float* out = P + ((long long)blockIdx.z * m + i) * n;
+                if (n % 4 == 0) {  // rows are 16-byte aligned
 #pragma unroll
-                for (int c = 0; c < 64; ++c)
-                    if (jb + c < n) out[jb + c] = sum[c];
+                    for (int c = 0; c < 64; c += 4)
+                        if (jb + c < n)
+                            *reinterpret_cast<float4*>(out + jb + c) =
+                                make_float4(sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 64; ++c)
+                        if (jb + c < n) out[jb + c] = sum[c];
+                }
             }
         }
     }
@@ -327,8 +337,8 @@ __global__ void __launch_bounds__(NTHR, 1)
                 mbar_arrive_expect_tx(&sm.full[b], 4 * 128 * TK * 4);
                 bulk_load(sm.a_hi[b], a_src, 128 * TK * 4, &sm.full[b]);
                 bulk_load(sm.a_lo[b], a_src + 128 * TK, 128 * TK * 4, &sm.full[b]);
-                bulk_load(sm.b_hi[b], b_src, 128 * TK * 4, &sm.full[b]);
-                bulk_load(sm.b_lo[b], b_src + 128 * TK, 128 * TK * 4, &sm.full[b]);
+                bulk_load(sm.b[b][0], b_src, 128 * TK * 4, &sm.full[b]);
+                bulk_load(sm.b[b][1], b_src + 128 * TK, 128 * TK * 4, &sm.full[b]);
                 if (++ks == nks) {
                     ks = 0;
                     tile += G;
@@ -367,8 +377,8 @@ __global__ void __launch_bounds__(NTHR, 1)
             if (p == 0) {  // C's images for this trial block and stage, by bulk copy
                 const float* src = Cimg + ((long long)((ctile % ntb) * nks + cks) * 2) * (128 * TK);
                 mbar_arrive_expect_tx(&sm.full[b], 2 * 128 * TK * 4);
-                bulk_load(sm.b_hi[b], src, 128 * TK * 4, &sm.full[b]);
-                bulk_load(sm.b_lo[b], src + 128 * TK, 128 * TK * 4, &sm.full[b]);
+                bulk_load(sm.b[b][0], src, 128 * TK * 4, &sm.full[b]);
+                bulk_load(sm.b[b][1], src + 128 * TK, 128 * TK * 4, &sm.full[b]);
             }
             unsigned char* ah = reinterpret_cast<unsigned char*>(sm.a_hi[b]);
             unsigned char* al = reinterpret_cast<unsigned char*>(sm.a_lo[b]);
