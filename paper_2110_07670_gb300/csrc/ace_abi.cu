@@ -560,6 +560,19 @@ int run_pairs(ace_plan* P, const R* fl, const R* fr, R* accl, R* accr, int symme
     return ACE_OK;
 }
 
+// The streamed tensor-core Gram's K-slice partials in the plan's scratch.
+int gram_partials(ace_plan* P, const float* A, int m, const float* B, int n, float** part, int* nchunk,
+                  cudaStream_t st) {
+    const long long K = 2LL * P->npw;
+    const long long kc = gram_stream_kchunk(m, n, K, P->sms, P->gram_kmax);
+    *nchunk = (int)((K + kc - 1) / kc);
+    // single-precision partials: half the doubles' room is enough
+    ACE_TRY(grow(&P->d_part, &P->part_cap, ((size_t)*nchunk * m * n + 1) / 2));
+    *part = reinterpret_cast<float*>(P->d_part);
+    ACE_CKL(launch_gram_stream(A, B, m, n, K, kc, *part, P->d_err, st));
+    return ACE_OK;
+}
+
 // G[i][j] = <A_i|B_j> (Gamma inner product), double [m][n].
 template <typename R>
 int gram(ace_plan* P, const cx<R>* A, int m, const cx<R>* B, int n, double* G, cudaStream_t st) {
@@ -567,12 +580,9 @@ int gram(ace_plan* P, const cx<R>* A, int m, const cx<R>* B, int n, double* G, c
     mark(P, PH_GRAM, st);
     if constexpr (sizeof(R) == 4) {
         if (P->tensor_gram) {
-            const long long kc = gram_stream_kchunk(m, n, K, P->sms, P->gram_kmax);
-            const int nchunk = (int)((K + kc - 1) / kc);
-            // single-precision partials: half the doubles' room is enough
-            ACE_TRY(grow(&P->d_part, &P->part_cap, ((size_t)nchunk * m * n + 1) / 2));
-            float* part = reinterpret_cast<float*>(P->d_part);
-            ACE_CKL(launch_gram_stream((const float*)A, (const float*)B, m, n, K, kc, part, P->d_err, st));
+            float* part;
+            int nchunk;
+            ACE_TRY(gram_partials(P, (const float*)A, m, (const float*)B, n, &part, &nchunk, st));
             ACE_CKL(launch_gram_finish_f32(part, nchunk, (const float*)A, (const float*)B, m, n, K, G, n, st));
             return ACE_OK;
         }
@@ -1077,20 +1087,28 @@ int scdm_impl(ace_plan* P, const void* psi_G, int n, int preselect, void* phi_G,
 
 template <typename R>
 int apply_impl(ace_plan* P, const void* xi, int n_occ, const void* psi, int T, void* out, cudaStream_t st) {
-    ACE_TRY(grow(&P->d_C, &P->C_cap, (size_t)T * n_occ));
-    ACE_TRY(gram<R>(P, (const cx<R>*)psi, T, (const cx<R>*)xi, n_occ, P->d_C, st));  // C[t][k] = <psi_t|xi_k>
-    mark(P, PH_XI, st);
     if constexpr (sizeof(R) == 4) {
-        if (P->tensor_gram) {  // -xi C on the tensor cores
+        if (P->tensor_gram) {  // C[t][k] = <psi_t|xi_k> as the product's operand image, then -xi C
+            const long long K = 2LL * P->npw;
+            float* part;
+            int nchunk;
+            mark(P, PH_GRAM, st);
             ACE_TRY(grow(&P->d_csplit, &P->csplit_cap, apply_product_scratch(T, n_occ)));
+            ACE_TRY(gram_partials(P, (const float*)psi, T, (const float*)xi, n_occ, &part, &nchunk, st));
+            ACE_CKL(launch_gram_finish_image(part, nchunk, (const float*)psi, (const float*)xi, T, n_occ, K,
+                                             P->d_csplit, st));
+            mark(P, PH_XI, st);
             // xi's split image, when ace_apply_prepare made one of this xi
             const float* ximg = P->ximg_src == xi && P->ximg_n == n_occ ? P->d_ximg : nullptr;
-            ACE_CKL(launch_apply_product(P->d_C, T, n_occ, (const float*)xi, 2LL * P->npw, P->d_csplit, (float*)out,
-                                         P->sms, P->d_err, st, ximg));
+            ACE_CKL(launch_apply_product(T, n_occ, (const float*)xi, K, P->d_csplit, (float*)out, P->sms, P->d_err, st,
+                                         ximg));
             mark(P, PH_IDLE, st);
             return ACE_OK;
         }
     }
+    ACE_TRY(grow(&P->d_C, &P->C_cap, (size_t)T * n_occ));
+    ACE_TRY(gram<R>(P, (const cx<R>*)psi, T, (const cx<R>*)xi, n_occ, P->d_C, st));  // C[t][k] = <psi_t|xi_k>
+    mark(P, PH_XI, st);
     ACE_CKL(launch_gemm_nn<R>(P->d_C, T, n_occ, (const R*)xi, 2LL * P->npw, -1.0, (R*)out, false, st));
     mark(P, PH_IDLE, st);
     return ACE_OK;
@@ -1101,9 +1119,23 @@ int apply_impl(ace_plan* P, const void* xi, int n_occ, const void* psi, int T, v
 template <typename R>
 int apply_energy_impl(ace_plan* P, const void* xi, int n_occ, const void* psi, int T, double* E, cudaStream_t st) {
     ACE_TRY(grow(&P->d_C, &P->C_cap, (size_t)T * n_occ));
-    ACE_TRY(gram<R>(P, (const cx<R>*)psi, T, (const cx<R>*)xi, n_occ, P->d_C, st));
-    mark(P, PH_ENERGY, st);
-    ACE_CKL(launch_sumsq(P->d_C, (long long)T * n_occ, -1.0, P->d_E, st));
+    bool done = false;
+    if constexpr (sizeof(R) == 4) {
+        if (P->tensor_gram) {  // squares summed per block of the Gram's finish (d_C: the block sums)
+            float* part;
+            int nchunk;
+            mark(P, PH_GRAM, st);
+            ACE_TRY(gram_partials(P, (const float*)psi, T, (const float*)xi, n_occ, &part, &nchunk, st));
+            ACE_CKL(launch_gram_finish_sumsq(part, nchunk, (const float*)psi, (const float*)xi, T, n_occ, 2LL * P->npw,
+                                             P->d_C, -1.0, P->d_E, st));
+            done = true;
+        }
+    }
+    if (!done) {
+        ACE_TRY(gram<R>(P, (const cx<R>*)psi, T, (const cx<R>*)xi, n_occ, P->d_C, st));
+        mark(P, PH_ENERGY, st);
+        ACE_CKL(launch_sumsq(P->d_C, (long long)T * n_occ, -1.0, P->d_E, st));
+    }
     mark(P, PH_IDLE, st);
     ACE_CK(cudaMemcpyAsync(&P->h_res->E, P->d_E, sizeof(double), cudaMemcpyDeviceToHost, st));
     ACE_CK(cudaStreamSynchronize(st));

@@ -230,12 +230,13 @@ long long gram_stream_kchunk(int m, int n, long long K, int sms, int max_k);
 cudaError_t launch_gram_stream(const float* A, const float* B, int m, int n, long long K, long long kchunk, float* P,
                                int* err, cudaStream_t st, bool absval = false);
 // out[t][j] = -sum_k C[t][k] xi[k][j] on tcgen05 (K psi = -xi C^T, Eq. 5):
-// C [T][n] double, xi [n][K] float, out [T][K] float; Cimg: scratch of
-// apply_product_scratch(T, n) floats (16-byte aligned) for C's TF32 split.
+// xi [n][K] float, out [T][K] float; Cimg: C [T][n]'s TF32 split as
+// launch_gram_finish_image writes it (apply_product_scratch(T, n) floats, 16-byte
+// aligned).
 // Ximg (or null): xi's split image from launch_xi_image, which feeds xi to the
 // tensor cores by bulk copies instead of the producer warps.
 size_t apply_product_scratch(int T, int n);
-cudaError_t launch_apply_product(const double* C, int T, int n, const float* xi, long long K, float* Cimg, float* out,
+cudaError_t launch_apply_product(int T, int n, const float* xi, long long K, const float* Cimg, float* out,
                                  int sms, int* err, cudaStream_t st, const float* Ximg = nullptr);
 // xi [n][K] float -> Ximg: xi_image_floats(n, K) floats (16-byte aligned), the
 // TF32 hi / lo split of xi^T in the product's swizzled operand tiles.
@@ -250,6 +251,13 @@ cudaError_t launch_overlap_finish(const PT* P, int nchunk, int m, double scale, 
 // launch_gram_finish for single-precision partials
 cudaError_t launch_gram_finish_f32(const float* P, int nchunk, const float* A, const float* B, int m, int n,
                                    long long K, double* G, int ldg, cudaStream_t st);
+// ... with the finished matrix written as the apply product's operand image
+// (img: apply_product_scratch(m, n) floats), or reduced to out = coef sum G^2
+// (part: m ceil(n / 32) doubles of scratch)
+cudaError_t launch_gram_finish_image(const float* P, int nchunk, const float* A, const float* B, int m, int n,
+                                     long long K, float* img, cudaStream_t st);
+cudaError_t launch_gram_finish_sumsq(const float* P, int nchunk, const float* A, const float* B, int m, int n,
+                                     long long K, double* part, double coef, double* out, cudaStream_t st);
 // G[i][j] = 2 sum_c P[c][i][j] - (A_i0 B_j0 + A_i1 B_j1)   (G = 0 counted once)
 template <typename R>
 cudaError_t launch_gram_finish(const double* P, int nchunk, const R* A, const R* B, int m, int n, long long K,

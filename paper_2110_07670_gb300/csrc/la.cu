@@ -3,6 +3,7 @@
 // exchange-energy reduction (arXiv:2110.07670 Section 2.2 and Eq. 4-5).
 #include "internal.h"
 #include "tma.cuh"
+#include "umma.cuh"
 
 namespace ace {
 
@@ -126,34 +127,78 @@ __global__ void gram_finish_kernel(const PT* __restrict__ P, int nchunk, const R
 }
 
 // The same from single-precision partials with many K slices: a block owns
-// 32 consecutive elements (one per lane) and its eight warps sum interleaved
-// eighths of the slices (four loads in flight each), combined in a fixed order.
+// 32 consecutive columns (one per lane) of one row and its eight warps sum
+// interleaved eighths of the slices (four loads in flight each), combined in a
+// fixed order.  A warp's sums are float-float (TwoSum, about 2^-46 of the sum of
+// magnitudes): converting and adding every partial in double kept the FP64 pipe
+// 71% busy (17 us for 144 slices of 128 x 128).  What the finished element G_ij
+// becomes:
+//   FIN_MATRIX  G[i][j]
+//   FIN_IMAGE   the apply product's operand image of C = G: TF32 hi / lo in the
+//               swizzled tiles of launch_apply_product, zero outside m x n (the
+//               grid covers the padded tiles)
+//   FIN_SUMSQ   sum over the block's columns of G_ij^2 (the fast MTS energy)
+enum GramFinish { FIN_MATRIX = 0, FIN_IMAGE = 1, FIN_SUMSQ = 2 };
+
+__device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
+    const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
+    hi = t;
+}
+
+template <int FIN>
 __global__ void __launch_bounds__(256) gram_finish_f32_kernel(const float* __restrict__ P, int nchunk,
                                                               const float* __restrict__ A,
                                                               const float* __restrict__ B, int m, int n, long long K,
-                                                              double* __restrict__ G, int ldg) {
+                                                              double* __restrict__ G, int ldg,
+                                                              float* __restrict__ img) {
     __shared__ double part[8][32];
     const long long tot = (long long)m * n;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long e = (long long)blockIdx.x * 32 + lane;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    if (e < tot) {
+    const int i = blockIdx.x, j = blockIdx.y * 32 + lane;
+    const bool in = i < m && j < n;
+    const long long e = (long long)i * n + j;
+    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    if (in) {
         int c = w;
         for (; c + 24 < nchunk; c += 32) {
+            float v[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) s[u] += (double)P[(long long)(c + 8 * u) * tot + e];
+            for (int u = 0; u < 4; ++u) v[u] = P[(long long)(c + 8 * u) * tot + e];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ff_add(hi[u], lo[u], v[u]);
         }
-        for (; c < nchunk; c += 8) s[0] += (double)P[(long long)c * tot + e];
+        for (; c < nchunk; c += 8) ff_add(hi[0], lo[0], P[(long long)c * tot + e]);
+#pragma unroll
+        for (int u = 1; u < 4; ++u) {
+            ff_add(hi[0], lo[0], hi[u]);
+            lo[0] = __fadd_rn(lo[0], lo[u]);
+        }
     }
-    part[w][lane] = (s[0] + s[1]) + (s[2] + s[3]);
+    part[w][lane] = (double)hi[0] + (double)lo[0];
     __syncthreads();
-    if (w == 0 && e < tot) {
-        double sum = 0.0;
-        for (int k = 0; k < 8; ++k) sum += part[k][lane];
-        const int i = (int)(e / n), j = (int)(e % n);
+    if (w != 0) return;
+    double g = 0.0;
+    if (in) {
+        for (int k = 0; k < 8; ++k) g += part[k][lane];
         const double g0 = double(A[(long long)i * K]) * double(B[(long long)j * K]) +
                           double(A[(long long)i * K + 1]) * double(B[(long long)j * K + 1]);
-        G[(long long)i * ldg + j] = 2.0 * sum - g0;
+        g = 2.0 * g - g0;
+    }
+    if constexpr (FIN == FIN_MATRIX) {
+        if (in) G[(long long)i * ldg + j] = g;
+    } else if constexpr (FIN == FIN_IMAGE) {
+        // tile (i / 128, blockIdx.y): rows of 32 values, 16-byte chunk c of row r at chunk c ^ (r % 8)
+        const int row = i & 127;
+        float* tile = img + ((long long)(i >> 7) * gridDim.y + blockIdx.y) * (2 * 128 * 32);
+        const int o = row * 32 + (lane ^ ((row & 7) << 2));
+        const float h = __uint_as_float(umma::tf32_round((float)g));
+        tile[o] = h;
+        tile[128 * 32 + o] = __uint_as_float(umma::tf32_round((float)(g - (double)h)));
+    } else {
+        double s = g * g;
+        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if (lane == 0) G[(long long)blockIdx.y * gridDim.x + blockIdx.x] = s;
     }
 }
 
@@ -367,13 +412,14 @@ __global__ void energy_final_kernel(const double* __restrict__ part, int nb, dou
     if (threadIdx.x == 0) *E = coef * s;
 }
 
-// out = coef * sum_k x[k]^2 in one block, a fixed order (the fast MTS energy
-// sum_t <psi_t|K psi_t> = -sum_{t,k} C_tk^2 from the apply's Gram C).
+// out = coef * sum_k x[k]^2 (or x[k]) in one block, a fixed order (the fast MTS
+// energy sum_t <psi_t|K psi_t> = -sum_{t,k} C_tk^2 from the apply's Gram C).
+template <bool SQUARE>
 __global__ void __launch_bounds__(1024) sumsq_kernel(const double* __restrict__ x, long long n, double coef,
                                                      double* __restrict__ out) {
     __shared__ double ws[32];
     double s = 0.0;
-    for (long long k = threadIdx.x; k < n; k += blockDim.x) s += x[k] * x[k];
+    for (long long k = threadIdx.x; k < n; k += blockDim.x) s += SQUARE ? x[k] * x[k] : x[k];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -507,8 +553,22 @@ template cudaError_t launch_overlap_finish<double>(const double*, int, int, doub
 
 cudaError_t launch_gram_finish_f32(const float* P, int nchunk, const float* A, const float* B, int m, int n,
                                    long long K, double* G, int ldg, cudaStream_t st) {
-    const long long tot = (long long)m * n;
-    gram_finish_f32_kernel<<<(unsigned)((tot + 31) / 32), 256, 0, st>>>(P, nchunk, A, B, m, n, K, G, ldg);
+    gram_finish_f32_kernel<FIN_MATRIX><<<dim3(m, (n + 31) / 32), 256, 0, st>>>(P, nchunk, A, B, m, n, K, G, ldg, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gram_finish_image(const float* P, int nchunk, const float* A, const float* B, int m, int n,
+                                     long long K, float* img, cudaStream_t st) {
+    gram_finish_f32_kernel<FIN_IMAGE><<<dim3((m + 127) / 128 * 128, (n + 31) / 32), 256, 0, st>>>(
+        P, nchunk, A, B, m, n, K, nullptr, 0, img);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gram_finish_sumsq(const float* P, int nchunk, const float* A, const float* B, int m, int n,
+                                     long long K, double* part, double coef, double* out, cudaStream_t st) {
+    const dim3 grid(m, (n + 31) / 32);
+    gram_finish_f32_kernel<FIN_SUMSQ><<<grid, 256, 0, st>>>(P, nchunk, A, B, m, n, K, part, 0, nullptr);
+    sumsq_kernel<false><<<1, 1024, 0, st>>>(part, (long long)grid.x * grid.y, coef, out);
     return cudaGetLastError();
 }
 
@@ -778,7 +838,7 @@ cudaError_t launch_neg_cholesky_inverse(const double* M, int n, double* L, doubl
 }
 
 cudaError_t launch_sumsq(const double* x, long long n, double coef, double* out, cudaStream_t st) {
-    sumsq_kernel<<<1, 1024, 0, st>>>(x, n, coef, out);
+    sumsq_kernel<true><<<1, 1024, 0, st>>>(x, n, coef, out);
     return cudaGetLastError();
 }
 

@@ -303,9 +303,9 @@ __global__ void __launch_bounds__(NTHR, 1)
 // handed out round-robin over the blocks (block b: tiles b, b + G, ...), the
 // trial blocks of one j range adjacent so the second reads xi from L2; the K
 // stages of 32 ACE vectors run on across tiles, and an accumulator turn never
-// spans two tiles.  C comes pre-split and pre-swizzled (Cimg: per trial block
-// and stage, the hi and lo shared-memory images of 16 KB each), so one bulk
-// copy per half fills a stage's B operand.  Producer thread p owns, in every
+// spans two tiles.  C comes pre-split and pre-swizzled (Cimg, written by the
+// Gram's finish: per trial block and stage, the hi and lo shared-memory images of
+// 16 KB each), so one bulk copy per half fills a stage's B operand.  Producer thread p owns, in every
 // stage, xi[k0 + 4 u + (p / 8) % 4][j0 + 16 (p / 32) + 2 (p % 8) + {0, 1}]
 // (u = 0..7: a warp covers 4 rows of 16 reals).
 // IMG: xi comes as Ximg, its TF32 hi / lo images per 128-real tile and stage
@@ -462,30 +462,6 @@ __global__ void __launch_bounds__(NTHR, 1)
     if (warp == 0) umma::tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// C [T][n] (double) split to TF32 hi / lo and laid out as the product's B
-// operand images: Cimg[tb][ks][hi, lo][128 x 32 in the 128-byte swizzle
-// layout], trials t = 128 tb + row, ACE vectors k = 32 ks + column; zero
-// outside T x n.
-__global__ void split_c_kernel(const double* __restrict__ C, int T, int n, int nks, float* __restrict__ Cimg) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // one (tb, ks, row, column)
-    const int ntb = (T + 127) / 128;
-    if (e >= (long long)ntb * nks * 128 * TK) return;
-    const int col = (int)(e % TK), row = (int)((e / TK) % 128);
-    const long long blk = e / (128 * TK);
-    const int ks = (int)(blk % nks), tb = (int)(blk / nks);
-    const int t = tb * 128 + row, k = ks * TK + col;
-    float h = 0.f, l = 0.f;
-    if (t < T && k < n) {
-        const double c = C[(long long)t * n + k];
-        h = __uint_as_float(umma::tf32_round((float)c));
-        l = __uint_as_float(umma::tf32_round((float)(c - (double)h)));
-    }
-    float* img = Cimg + blk * 2 * (128 * TK);
-    const uint32_t o = umma::sw128_offset(row, col) / 4;
-    img[o] = h;
-    img[128 * TK + o] = l;
-}
-
 // Ximg[jt][ks][hi, lo][128 x TK swizzled]: the TF32 split of xi^T's tile of
 // reals jt * 128 .. + 127 and ACE vectors ks * TK .. + TK - 1, in the K-major
 // 128-byte swizzle layout the product's A operand takes (zero past K and n).
@@ -561,14 +537,12 @@ cudaError_t launch_xi_image(const float* xi, int n, long long K, float* Ximg, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_apply_product(const double* C, int T, int n, const float* xi, long long K, float* Cimg, float* out,
-                                 int sms, int* err, cudaStream_t st, const float* Ximg) {
+cudaError_t launch_apply_product(int T, int n, const float* xi, long long K, const float* Cimg, float* out, int sms,
+                                 int* err, cudaStream_t st, const float* Ximg) {
     if (K % 2 != 0 || ((uintptr_t)xi % 8) || ((uintptr_t)out % 8) || ((uintptr_t)Cimg % 16) ||
         ((uintptr_t)Ximg % 16))
         return cudaErrorInvalidValue;
     const int nks = (n + TK - 1) / TK;
-    const long long tot = (long long)((T + 127) / 128) * nks * 128 * TK;
-    split_c_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(C, T, n, nks, Cimg);
     const void* k = Ximg ? (const void*)apply_product<true> : (const void*)apply_product<false>;
     cudaError_t e = set_smem(k, st);
     if (e != cudaSuccess) return e;
