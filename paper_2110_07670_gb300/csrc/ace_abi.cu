@@ -102,6 +102,9 @@ struct ace_plan {
     int npw = 0;
     int* d_ip = nullptr;
     int* d_in = nullptr;
+    bool sphere = false;       // orbital and W z transforms over the sphere's pencils only (generic.cuh)
+    int* d_sphere = nullptr;   // its tables: offsets [n1 n2 + 1], entries (int2, 8-byte aligned), units
+    SphereArgs sp{};
     AxisPlan ax[3];
     void* d_tw[3] = {nullptr, nullptr, nullptr};
     int* d_freq[3] = {nullptr, nullptr, nullptr};
@@ -405,9 +408,15 @@ int run_to_real(ace_plan* P, const cx<R>* psi, const Quad* dq, int ntrans, R* ou
     for (int t0 = 0; t0 < ntrans; t0 += P->batch) {
         const int nb = std::min(P->batch, ntrans - t0);
         a.t0 = t0;
-        ACE_CK(cudaMemsetAsync(spec, 0, (size_t)nb * P->N * sizeof(cx<R>), st));
-        ACE_CKL(launch_scatter<R>(psi, dq, t0, nb, P->npw, P->d_ip, P->d_in, spec, P->N, st));
-        ACE_CKL(launch_pass<R>(a, P->s_z, PRO_LOAD, EPI_STORE, MID_NONE, +1, nb, st));
+        if (P->sphere) {
+            SphereArgs sp = P->sp;
+            sp.psi = psi;
+            ACE_CKL(sphere_launch(a, sp, true, nb, st));
+        } else {
+            ACE_CK(cudaMemsetAsync(spec, 0, (size_t)nb * P->N * sizeof(cx<R>), st));
+            ACE_CKL(launch_scatter<R>(psi, dq, t0, nb, P->npw, P->d_ip, P->d_in, spec, P->N, st));
+            ACE_CKL(launch_pass<R>(a, P->s_z, PRO_LOAD, EPI_STORE, MID_NONE, +1, nb, st));
+        }
         if (P->fused_xy) {
             ACE_CKL(launch_pass<R>(a, P->s_xy, PRO_LOAD, EPI_SPLIT, MID_NONE, +1, nb, st));
         } else {
@@ -435,7 +444,10 @@ int run_to_recip(ace_plan* P, const R* acc, const Quad* dq, int ntrans, double s
             ACE_CKL(launch_pass<R>(a, P->s_x, PRO_PACK2, EPI_STORE, MID_NONE, -1, nb, st));
             ACE_CKL(launch_pass<R>(a, P->s_y, PRO_LOAD, EPI_STORE, MID_NONE, -1, nb, st));
         }
-        ACE_CKL(launch_pass<R>(a, P->s_z, PRO_LOAD, EPI_STORE, MID_NONE, -1, nb, st));
+        if (P->sphere)
+            ACE_CKL(sphere_launch(a, P->sp, false, nb, st));
+        else
+            ACE_CKL(launch_pass<R>(a, P->s_z, PRO_LOAD, EPI_STORE, MID_NONE, -1, nb, st));
         ACE_CKL(launch_gather<R>(spec, dq, t0, nb, P->npw, P->d_ip, P->d_in, P->N, s, out, st));
     }
     return ACE_OK;
@@ -1154,7 +1166,7 @@ void free_plan(ace_plan* P) {
     for (auto s2 : P->aux) cudaStreamDestroy(s2);
     for (auto e : P->aux_ev) cudaEventDestroy(e);
     if (P->fork_ev) cudaEventDestroy(P->fork_ev);
-    void* ptrs[] = {P->d_ip, P->d_in, P->d_tw[0], P->d_tw[1], P->d_tw[2], P->d_freq[0], P->d_freq[1], P->d_freq[2], P->d_phi, P->d_acc, P->d_spec,
+    void* ptrs[] = {P->d_ip, P->d_in, P->d_sphere, P->d_tw[0], P->d_tw[1], P->d_tw[2], P->d_freq[0], P->d_freq[1], P->d_freq[2], P->d_phi, P->d_acc, P->d_spec,
                     P->d_WG, P->d_M, P->d_S, P->d_L, P->d_Linv, P->d_chol, P->d_E, P->d_status, P->d_err, P->d_part, P->d_quads,
                     P->d_epart, P->d_tphi, P->d_tacc, P->d_C, P->d_kern, P->d_kern_t, P->d_kern_r, P->d_pipe, P->d_csplit, P->d_ximg,
                     P->scdm.gv, P->scdm.dpsi, P->scdm.dens, P->scdm.isel, P->scdm.A, P->scdm.nu,
@@ -1568,6 +1580,37 @@ int create_impl(ace_plan* P, const ace_opts* opts) {
     ACE_TRY(dalloc((void**)&P->d_in, P->npw * sizeof(int)));
     ACE_CK(cudaMemcpy(P->d_ip, ip.data(), P->npw * sizeof(int), cudaMemcpyHostToDevice));
     ACE_CK(cudaMemcpy(P->d_in, in.data(), P->npw * sizeof(int), cudaMemcpyHostToDevice));
+    P->sphere = sizeof(R) == 4 && P->fused_xy && generic_supported(P->n[0], P->n[1], P->n[2], 226 * 1024);
+    if (P->sphere) {
+        // pencil (plane position) -> its plane waves, +G and -G
+        const int plane = P->n[1] * P->n[2], unit = sphere_unit(P->n[1], P->n[2]);
+        std::vector<int> off(plane + 1, 0);
+        for (int p = 0; p < P->npw; ++p) {
+            ++off[ip[p] % plane + 1];
+            if (in[p] != ip[p]) ++off[in[p] % plane + 1];
+        }
+        for (int k = 0; k < plane; ++k) off[k + 1] += off[k];
+        std::vector<int> at(off.begin(), off.end() - 1), ent(2 * (size_t)off[plane]), list;
+        auto add = [&](int pos, int code) {
+            const int k = at[pos % plane]++;
+            ent[2 * (size_t)k] = pos / plane;
+            ent[2 * (size_t)k + 1] = code;
+        };
+        for (int p = 0; p < P->npw; ++p) {
+            add(ip[p], p);
+            if (in[p] != ip[p]) add(in[p], ~p);
+        }
+        for (int k = 0; k < plane; k += unit)
+            if (off[k + unit] > off[k]) list.push_back(k / unit);
+        const size_t n_off = (size_t)(plane + 2) / 2 * 2;  // entries stay 8-byte aligned
+        ACE_TRY(dalloc((void**)&P->d_sphere, (n_off + ent.size() + list.size()) * sizeof(int)));
+        ACE_CK(cudaMemcpy(P->d_sphere, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
+        ACE_CK(cudaMemcpy(P->d_sphere + n_off, ent.data(), ent.size() * sizeof(int), cudaMemcpyHostToDevice));
+        ACE_CK(cudaMemcpy(P->d_sphere + n_off + ent.size(), list.data(), list.size() * sizeof(int),
+                          cudaMemcpyHostToDevice));
+        P->sp = SphereArgs{P->d_sphere, reinterpret_cast<const int2*>(P->d_sphere + n_off),
+                           P->d_sphere + n_off + ent.size(), (int)list.size(), nullptr, P->npw};
+    }
     int ntrans_min = (P->n_occ_max + 1) / 2;
     int batch = opts && opts->pair_batch > 0 ? opts->pair_batch
                                              : (int)std::max<long long>(1, (512LL << 20) / (P->N * (long long)sizeof(cx<R>)));

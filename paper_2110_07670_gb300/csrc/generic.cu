@@ -50,6 +50,18 @@ cudaError_t launch_pencils(const PassArgs& a, int batch, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <typename V>
+cudaError_t launch_sphere(const PassArgs& a, const SphereArgs& sp, bool inverse, int batch, cudaStream_t st) {
+    const int units = a.n1 * a.n2 / (int)(sizeof(V) / 4), U = Units<V>::U;
+    const size_t smem = pencil_smem(a.n0);
+    auto k = inverse ? sphere_inverse<V> : sphere_forward<V>;
+    cudaError_t e = prepare(k, smem, st);
+    if (e != cudaSuccess) return e;
+    const int items = inverse ? units : sp.nlist;
+    k<<<dim3((unsigned)((items + U - 1) / U), (unsigned)batch), 32, smem, st>>>(a, units, sp);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 bool generic_supported(int n0, int n1, int n2, size_t smem_limit) {
@@ -72,6 +84,13 @@ cudaError_t generic_pencil_launch(const PassArgs& a, int mode, int batch, cudaSt
     }
     if (mode == 0) return launch_pencils<float, 0>(a, batch, st);
     return mode < 0 ? launch_pencils<float, -1>(a, batch, st) : launch_pencils<float, +1>(a, batch, st);
+}
+
+int sphere_unit(int n1, int n2) { return (long long)n1 * n2 % 2 == 0 ? 2 : 1; }
+
+cudaError_t sphere_launch(const PassArgs& a, const SphereArgs& sp, bool inverse, int batch, cudaStream_t st) {
+    return sphere_unit(a.n1, a.n2) == 2 ? launch_sphere<f2>(a, sp, inverse, batch, st)
+                                        : launch_sphere<float>(a, sp, inverse, batch, st);
 }
 
 }  // namespace ace

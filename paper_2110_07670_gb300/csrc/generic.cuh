@@ -481,5 +481,104 @@ __global__ void __launch_bounds__(32) pencils(PassArgs a, int units) {
         for (int z = h; z < n; z += L) dst[(long long)z * units] = turn_unit(col[z * U]);
 }
 
+// ------------------------------------------------- pencils of the sphere
+// The z transforms of the orbitals and of W touch the cutoff sphere only: of the
+// plane's pencils about a quarter hold plane waves.  off[p] .. off[p + 1] are
+// the entries of pencil p, each {z position, plane wave i for +G or ~i for -G}.
+
+// Orbitals to half-real space: the coefficients of a quad's two orbitals
+// (Z(G) = c_a + i c_b, Z(-G) = c_a^* + i c_b^*) gathered into shared columns,
+// inverse z, to the box; groups without plane waves only write zeros.  Replaces
+// a cleared box, a scatter and a z pass over it (334 us per 64 transforms of
+// 96^3); bound by the box's writes.
+template <typename V>
+__global__ void __launch_bounds__(32) sphere_inverse(PassArgs a, int units, SphereArgs sp) {
+    constexpr int U = Units<V>::U, L = Units<V>::L, W = sizeof(V) / 4;
+    extern __shared__ __align__(16) unsigned char smem_gen[];
+    cx<V>* buf = reinterpret_cast<cx<V>*>(smem_gen);
+    cx<float>* tw = reinterpret_cast<cx<float>*>(buf + a.n0 * U);
+    const int lane = threadIdx.x, l = lane % U, h = lane / U, n = a.n0;
+    const int p = blockIdx.x * U + l, t = blockIdx.y;
+    const bool on = p < units;
+    cx<V>* dst = reinterpret_cast<cx<V>*>(reinterpret_cast<cx<float>*>(a.dst) + t * a.dst_tstride) + p;
+    const int e0 = on ? sp.off[p * W] : 0, e2 = on ? sp.off[p * W + W] : 0, e1 = on ? sp.off[p * W + 1] : 0;
+    cx<V> zero;
+    zero.re = zero.im = V(0.0);
+    if (!__any_sync(0xffffffffu, e2 > e0)) {
+        if (on)
+            for (int z = h; z < n; z += L) dst[(long long)z * units] = zero;
+        return;
+    }
+    const Quad q = a.quads[a.t0 + t];
+    for (int j = lane; j < n; j += 32) tw[j] = reinterpret_cast<const cx<float>*>(a.twz)[j];
+    for (int z = h; z < n; z += L) buf[z * U + l] = zero;
+    __syncwarp();
+    const cx<float>* pa = reinterpret_cast<const cx<float>*>(sp.psi) + (long long)q.a * sp.npw;
+    const cx<float>* pb = reinterpret_cast<const cx<float>*>(sp.psi) + (long long)(q.c >= 0 ? q.c : q.a) * sp.npw;
+    for (int e = e0 + h; e < e2; e += L) {
+        const int2 en = sp.ent[e];
+        const bool neg = en.y < 0;
+        const int i = neg ? ~en.y : en.y;
+        const cx<float> ca = pa[i], cb = q.c >= 0 ? pb[i] : mk(0.f, 0.f);
+        const cx<float> v = neg ? mk(ca.re + cb.im, cb.re - ca.im) : mk(ca.re - cb.im, ca.im + cb.re);
+        float* u = reinterpret_cast<float*>(buf + en.x * U + l);
+        const int w = e >= e1 ? W - 1 : 0;
+        u[w] = v.re;
+        u[W + w] = v.im;
+    }
+    __syncwarp();
+    const AxisPlan& P = a.pz;
+    const int hh = e2 > e0 ? h : n;  // columns without plane waves stay zero
+    int Lb = 1;
+    for (int s = P.nstages - 1; s >= 0; --s) {
+        Lb *= P.radix[s];
+        with_radix(P.radix[s], [&](auto r) { pencil_stage<decltype(r)::value, +1, V>(buf + l, n, Lb, tw, hh); });
+    }
+    if (on)
+#pragma unroll 4
+        for (int z = h; z < n; z += L) dst[(long long)z * units] = turn_unit(buf[z * U + l]);
+}
+
+// The forward z transform of the pencils (units sp.list[0 .. nlist)) that hold
+// plane waves; only those entries of the box are written (in place).
+template <typename V>
+__global__ void __launch_bounds__(32) sphere_forward(PassArgs a, int units, SphereArgs sp) {
+    constexpr int U = Units<V>::U, L = Units<V>::L, W = sizeof(V) / 4;
+    extern __shared__ __align__(16) unsigned char smem_gen[];
+    cx<V>* buf = reinterpret_cast<cx<V>*>(smem_gen);
+    cx<float>* tw = reinterpret_cast<cx<float>*>(buf + a.n0 * U);
+    const int lane = threadIdx.x, l = lane % U, h = lane / U, n = a.n0;
+    const int g = blockIdx.x * U + l, t = blockIdx.y;
+    const bool on = g < sp.nlist;
+    const int p = on ? sp.list[g] : 0;
+    cx<float>* box = reinterpret_cast<cx<float>*>(a.dst) + t * a.dst_tstride;
+    const cx<V>* src = reinterpret_cast<const cx<V>*>(reinterpret_cast<const cx<float>*>(a.src) + t * a.src_tstride) + p;
+    if (on)
+#pragma unroll 4
+        for (int z = h; z < n; z += L) async_unit(buf + z * U + l, src + (long long)z * units);
+    for (int j = lane; j < n; j += 32) tw[j] = reinterpret_cast<const cx<float>*>(a.twz)[j];
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    if (W == 2) {
+        if (on)
+            for (int z = h; z < n; z += L) buf[z * U + l] = turn_unit(buf[z * U + l]);
+        __syncwarp();
+    }
+    const AxisPlan& P = a.pz;
+    const int hh = on ? h : n;
+    int Lb = n;
+    for (int s = 0; s < P.nstages; ++s) {
+        with_radix(P.radix[s], [&](auto r) { pencil_stage<decltype(r)::value, -1, V>(buf + l, n, Lb, tw, hh); });
+        Lb /= P.radix[s];
+    }
+    if (!on) return;
+    const int e0 = sp.off[p * W], e1 = sp.off[p * W + 1], e2 = sp.off[p * W + W];
+    for (int e = e0 + h; e < e2; e += L) {
+        const int z = sp.ent[e].x, w = e >= e1 ? W - 1 : 0;
+        const float* u = reinterpret_cast<const float*>(buf + z * U + l);
+        box[(long long)z * units * W + p * W + w] = mk(u[w], u[W + w]);
+    }
+}
+
 }  // namespace generic_detail
 }  // namespace ace

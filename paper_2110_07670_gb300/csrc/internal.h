@@ -198,6 +198,21 @@ bool generic_supported(int n0, int n1, int n2, size_t smem_limit);
 cudaError_t generic_plane_launch(const PassArgs& a, int pro, int epi, int batch, cudaStream_t st);
 cudaError_t generic_pencil_launch(const PassArgs& a, int mode, int batch, cudaStream_t st);
 
+// The z transforms of orbitals and W over the cutoff sphere's pencils only
+// (generic.cuh, single precision): the plan's tables ...
+struct SphereArgs {
+    const int* off;    // [n1 n2 + 1] entries of every plane position
+    const int2* ent;   // {z position, plane wave i (+G) or ~i (-G)}
+    const int* list;   // units (sphere_unit neighbouring pencils) with entries
+    int nlist;
+    const void* psi;   // inverse: half-sphere coefficients [*][npw]
+    int npw;
+};
+int sphere_unit(int n1, int n2);  // pencils per unit: 2 where a z row holds an even count
+// ... inverse: the quads' orbitals gathered, inverse z, the whole box written;
+// forward: the box's listed pencils forward z, their sphere entries written back.
+cudaError_t sphere_launch(const PassArgs& a, const SphereArgs& sp, bool inverse, int batch, cudaStream_t st);
+
 // Launch one pass over `batch` transforms (gridDim.y) of the box.
 template <typename R>
 cudaError_t launch_pass(const PassArgs& a, const PassShape& s, int pro, int epi, int mid, int sgn, int batch,
