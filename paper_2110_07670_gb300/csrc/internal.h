@@ -348,7 +348,7 @@ size_t neg_cholesky_work(int n);
 cudaError_t launch_neg_cholesky_blocked(const double* M, int n, double* L, double* Linv, int* status, double* work,
                                         int* nlaunch, cudaStream_t st);
 
-// Cholesky of -M and the inverse of its factor, in double, one thread block.
+// Cholesky of -M and the inverse of its factor, in double, one thread block (n <= 64).
 // status: 0 ok, 1 not positive definite.
 cudaError_t launch_neg_cholesky_inverse(const double* M, int n, double* L, double* Linv, int* status,
                                         cudaStream_t st);

@@ -302,47 +302,71 @@ __global__ void __launch_bounds__(256) gemm_nn_kernel(const double* __restrict__
 }
 
 // ------------------------------------------------ Cholesky and inverse (FP64)
-// -M = L L^T (right-looking, one block), then Linv = L^-1 column by column.
-
-__global__ void __launch_bounds__(1024) neg_cholesky_inverse_kernel(const double* __restrict__ M, int n,
-                                                                     double* __restrict__ L,
-                                                                     double* __restrict__ Linv,
-                                                                     int* __restrict__ status) {
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    // lower triangle of -M, symmetrised
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e % n;
-        L[e] = i >= j ? -0.5 * (M[(long long)i * n + j] + M[(long long)j * n + i]) : 0.0;
-    }
-    __syncthreads();
+// A = L L^T (lower triangle of A in, L out) and X = L^-1 (identity in) of an
+// n x n tile in shared memory, by the whole block: step k takes the pivot's root
+// (one thread its reciprocal, another the root itself), scales column k of A and
+// row k of X, and updates the trailing triangle of A and the rows of X below
+// with one pass.  X grows with the factorisation, so no column waits for a
+// chain of its own: a separate forward substitution with one column per thread
+// (64 orbitals 222 us, 27 59 us, 8 15 us; the 32 x 32 diagonal blocks of the
+// blocked factorisation 110 us each) was bound by that chain.  The bound left is
+// one SM's FP64 rate (two multiply-adds per cycle) and the pivots' latency.
+__device__ __forceinline__ void chol_inverse_tile(double* A, double* X, int n, int ld, double* piv, int* bad) {
     for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            const double d = L[(long long)k * n + k];
-            if (!(d > 0.0)) bad = 1;
-            L[(long long)k * n + k] = d > 0.0 ? sqrt(d) : 1.0;
+        if (threadIdx.x == 0 || threadIdx.x == 32) {
+            double dk = A[k * ld + k];
+            if (!(dk > 0.0)) {
+                *bad = 1;
+                dk = 1.0;
+            }
+            if (threadIdx.x == 0)
+                piv[0] = sqrt(dk);
+            else
+                piv[1] = 1.0 / sqrt(dk);
         }
         __syncthreads();
-        const double dkk = L[(long long)k * n + k];
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) L[(long long)i * n + k] /= dkk;
+        const double inv = piv[1];
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            if (i > k) A[i * ld + k] *= inv;
+            if (i <= k) X[k * ld + i] *= inv;
+        }
+        if (threadIdx.x == 0) A[k * ld + k] = piv[0];
         __syncthreads();
         const int m = n - k - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            const int i = k + 1 + e / m, j = k + 1 + e % m;
-            if (j <= i) L[(long long)i * n + j] -= L[(long long)i * n + k] * L[(long long)j * n + k];
+        for (int e = threadIdx.x; e < m * n; e += blockDim.x) {
+            const int r = e / n, i = k + 1 + r, j = e - r * n;
+            const double lik = A[i * ld + k];
+            if (j <= k)
+                X[i * ld + j] -= lik * X[k * ld + j];
+            else if (j <= i)
+                A[i * ld + j] -= lik * A[j * ld + k];
         }
         __syncthreads();
     }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        for (int i = 0; i < j; ++i) Linv[(long long)i * n + j] = 0.0;
-        Linv[(long long)j * n + j] = 1.0 / L[(long long)j * n + j];
-        for (int i = j + 1; i < n; ++i) {
-            double s = 0.0;
-            for (int k = j; k < i; ++k) s += L[(long long)i * n + k] * Linv[(long long)k * n + j];
-            Linv[(long long)i * n + j] = -s / L[(long long)i * n + i];
-        }
+}
+
+// -M = L L^T and L^-1 in one block (n <= 64), L and L^-1 with zero upper triangles.
+__global__ void __launch_bounds__(512) neg_cholesky_inverse_kernel(const double* __restrict__ M, int n,
+                                                                    double* __restrict__ L, double* __restrict__ Linv,
+                                                                    int* __restrict__ status) {
+    extern __shared__ double sm[];
+    __shared__ double piv[2];
+    __shared__ int bad;
+    const int ld = n | 1;
+    double *A = sm, *X = sm + n * ld;
+    if (threadIdx.x == 0) bad = 0;
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+        const int i = e / n, j = e - i * n;
+        A[i * ld + j] = i >= j ? -0.5 * (M[(long long)i * n + j] + M[(long long)j * n + i]) : 0.0;
+        X[i * ld + j] = i == j ? 1.0 : 0.0;
     }
     __syncthreads();
+    chol_inverse_tile(A, X, n, ld, piv, &bad);
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+        const int i = e / n, j = e - i * n;
+        L[e] = A[i * ld + j];
+        Linv[e] = X[i * ld + j];
+    }
     if (threadIdx.x == 0) *status = bad;
 }
 
@@ -428,55 +452,6 @@ __global__ void __launch_bounds__(1024) sumsq_kernel(const double* __restrict__ 
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
         *out = coef * t;
     }
-}
-
-// -M = L L^T and L^-1 with both in shared memory (n^2 doubles, n <= 160):
-// right-looking Cholesky in place, L copied out, then L^-1 in the same
-// buffer, one column per thread, reading L back through L1.
-__global__ void __launch_bounds__(1024) neg_cholesky_inverse_smem_kernel(const double* __restrict__ M, int n,
-                                                                          double* __restrict__ L,
-                                                                          double* __restrict__ Linv,
-                                                                          int* __restrict__ status) {
-    extern __shared__ double A[];
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e % n;
-        A[e] = i >= j ? -0.5 * (M[(long long)i * n + j] + M[(long long)j * n + i]) : 0.0;
-    }
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            const double d = A[k * n + k];
-            if (!(d > 0.0)) bad = 1;
-            A[k * n + k] = d > 0.0 ? sqrt(d) : 1.0;
-        }
-        __syncthreads();
-        const double dkk = A[k * n + k];
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) A[i * n + k] /= dkk;
-        __syncthreads();
-        const int m = n - k - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            const int i = k + 1 + e / m, j = k + 1 + e % m;
-            if (j <= i) A[i * n + j] -= A[i * n + k] * A[j * n + k];
-        }
-        __syncthreads();
-    }
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) L[e] = A[e];
-    __syncthreads();
-    // column j of L^-1 by forward substitution, kept in A's column j
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        for (int i = 0; i < j; ++i) A[i * n + j] = 0.0;
-        A[j * n + j] = 1.0 / L[(long long)j * n + j];
-        for (int i = j + 1; i < n; ++i) {
-            double s = 0.0;
-            for (int k = j; k < i; ++k) s += L[(long long)i * n + k] * A[k * n + j];
-            A[i * n + j] = -s / L[(long long)i * n + i];
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) Linv[e] = A[e];
-    if (threadIdx.x == 0) *status = bad;
 }
 
 // One block waits (bounded) on an mbarrier that expects 16 bytes no copy
@@ -683,45 +658,25 @@ __global__ void chol_init_kernel(const double* __restrict__ M, int n, int np, do
     X[e] = 0.0;
 }
 
-__global__ void __launch_bounds__(1024) chol_diag_kernel(double* __restrict__ W, int np, int k,
-                                                         double* __restrict__ T, int* __restrict__ status) {
-    __shared__ double a[CB][CB + 1], t[CB][CB + 1];
-    const int r = threadIdx.x / CB, c = threadIdx.x % CB;
+__global__ void __launch_bounds__(512) chol_diag_kernel(double* __restrict__ W, int np, int k,
+                                                        double* __restrict__ T, int* __restrict__ status) {
+    __shared__ double a[CB * (CB + 1)], t[CB * (CB + 1)], piv[2];
+    __shared__ int bad;
     double* blk = W + (long long)(k * CB) * np + k * CB;
-    a[r][c] = blk[(long long)r * np + c];
-    __syncthreads();
-    for (int p = 0; p < CB; ++p) {
-        if (threadIdx.x == 0) {
-            double d = a[p][p];
-            if (!(d > 0.0)) {
-                atomicExch(status, 1);
-                d = 1.0;
-            }
-            a[p][p] = sqrt(d);
-        }
-        __syncthreads();
-        if (r > p && c == p) a[r][p] /= a[p][p];
-        __syncthreads();
-        if (r > p && c > p && c <= r) a[r][c] -= a[r][p] * a[c][p];
-        __syncthreads();
-    }
-    blk[(long long)r * np + c] = c <= r ? a[r][c] : 0.0;
-    if (threadIdx.x < CB) {  // column c of the inverse of the lower-triangular factor
-        const int col = threadIdx.x;
-        for (int i = 0; i < CB; ++i) {
-            if (i < col) {
-                t[i][col] = 0.0;
-            } else if (i == col) {
-                t[i][col] = 1.0 / a[i][i];
-            } else {
-                double s = 0.0;
-                for (int j = col; j < i; ++j) s += a[i][j] * t[j][col];
-                t[i][col] = -s / a[i][i];
-            }
-        }
+    if (threadIdx.x == 0) bad = 0;
+    for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
+        const int r = e / CB, c = e % CB;
+        a[r * (CB + 1) + c] = blk[(long long)r * np + c];
+        t[r * (CB + 1) + c] = r == c ? 1.0 : 0.0;
     }
     __syncthreads();
-    T[(long long)k * CB * CB + r * CB + c] = t[r][c];
+    chol_inverse_tile(a, t, CB, CB + 1, piv, &bad);
+    for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
+        const int r = e / CB, c = e % CB;
+        blk[(long long)r * np + c] = c <= r ? a[r * (CB + 1) + c] : 0.0;
+        T[(long long)k * CB * CB + e] = t[r * (CB + 1) + c];
+    }
+    if (threadIdx.x == 0 && bad) atomicExch(status, 1);
 }
 
 __global__ void __launch_bounds__(1024) chol_panel_kernel(double* __restrict__ W, int np, int k,
@@ -807,7 +762,7 @@ cudaError_t launch_neg_cholesky_blocked(const double* M, int n, double* L, doubl
     chol_init_kernel<<<(unsigned)(((long long)np * np + 255) / 256), 256, 0, st>>>(M, n, np, W, X, status);
     ++count;
     for (int k = 0; k < nb; ++k) {
-        chol_diag_kernel<<<1, CB * CB, 0, st>>>(W, np, k, T, status);
+        chol_diag_kernel<<<1, 512, 0, st>>>(W, np, k, T, status);
         ++count;
         const int m = nb - k - 1;
         if (m > 0) {
@@ -825,15 +780,12 @@ cudaError_t launch_neg_cholesky_blocked(const double* M, int n, double* L, doubl
 
 cudaError_t launch_neg_cholesky_inverse(const double* M, int n, double* L, double* Linv, int* status,
                                         cudaStream_t st) {
-    const size_t smem = (size_t)n * n * sizeof(double);
-    if (smem <= 200 * 1024) {
-        static const cudaError_t attr = cudaFuncSetAttribute(
-            neg_cholesky_inverse_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (attr != cudaSuccess) return attr;
-        neg_cholesky_inverse_smem_kernel<<<1, 1024, smem, st>>>(M, n, L, Linv, status);
-    } else {
-        neg_cholesky_inverse_kernel<<<1, 1024, 0, st>>>(M, n, L, Linv, status);
-    }
+    const size_t smem = (size_t)2 * n * (n | 1) * sizeof(double);
+    static const cudaError_t attr = cudaFuncSetAttribute(neg_cholesky_inverse_kernel,
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+    if (attr != cudaSuccess) return attr;
+    if (n > 64) return cudaErrorInvalidValue;
+    neg_cholesky_inverse_kernel<<<1, n <= 16 ? 128 : 512, smem, st>>>(M, n, L, Linv, status);
     return cudaGetLastError();
 }
 
