@@ -194,9 +194,12 @@ struct ace_plan {
     int last_n_occ = 0;
     int pending_n_occ = 0;
     struct Result {
-        int status;
+        int status, err;
         double E;
     };
+    void* h_gamma = nullptr;  // pinned: the G = 0 coefficients of a call's vectors (gamma_begin)
+    size_t hg_cap = 0;
+    cudaEvent_t gamma_ev = nullptr;
     Result* h_res = nullptr;  // pinned host slots for the asynchronous build result
     Quad* h_quads = nullptr;  // pinned staging of the quads
     size_t hq_cap = 0;
@@ -339,7 +342,7 @@ int setup_shapes(ace_plan* P) {
     }
     // single precision: the runtime-size kernels take every box they can hold
     // (measured against the tile passes: see generic.cuh)
-    if (sizeof(R) == 4 && generic_supported(n0, n1, n2, (size_t)smax - 2048)) {
+    if (sizeof(R) == 4 && generic_supported(n0, n1, n2)) {
         P->gen = P->fused_xy = true;
         P->s_xy = mk_shape(1, n1, n2, 3);
         P->s_xy.gen = P->s_z.gen = 1;
@@ -536,14 +539,14 @@ int run_pairs(ace_plan* P, const R* fl, const R* fr, R* accl, R* accr, int symme
         return ACE_OK;
     }
     const int S = std::min(P->pair_streams, P->batch);
-    if (S <= 1 || ntrans <= 0) {
+    const int b = std::max(1, std::min(P->pair_sub > 0 ? P->pair_sub : P->batch / std::max(S, 1), P->batch / std::max(S, 1)));
+    if (S <= 1 || ntrans <= b) {  // one sub-batch has nothing to overlap with
         for (int t0 = 0; t0 < ntrans; t0 += P->batch) {
             a.t0 = t0;
             ACE_TRY(pair_batch<R>(P, a, std::min(P->batch, ntrans - t0), st, 0));
         }
         return ACE_OK;
     }
-    const int b = std::max(1, std::min(P->pair_sub > 0 ? P->pair_sub : P->batch / S, P->batch / S));
     while ((int)P->aux.size() < S) {
         cudaStream_t s2;
         cudaEvent_t e2;
@@ -698,28 +701,62 @@ void pack_pairs_blocked(int n, const std::vector<int>& pa, const std::vector<int
     }
 }
 
-// A bounded device-side wait that gave up leaves a flag; report and clear it.
+// Wait for the stream; a bounded device-side wait that gave up leaves a flag,
+// which comes back with the same wait: report and clear it.
 int check_device_error(ace_plan* P, cudaStream_t st) {
-    int err = 0;
-    ACE_CK(cudaMemcpyAsync(&err, P->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    ACE_CK(cudaMemcpyAsync(&P->h_res->err, P->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     ACE_CK(cudaStreamSynchronize(st));
-    if (err) {
+    if (P->h_res->err) {
         ACE_CK(cudaMemsetAsync(P->d_err, 0, sizeof(int), st));
         return fail(ACE_ERR_TIMEOUT, "a bounded wait for a bulk copy timed out on the device");
     }
     return ACE_OK;
 }
 
+// The Gamma-point check of vectors (Im c(0) = 0) in two halves, so that the
+// copy travels behind work that touches only the plan's scratch: gamma_begin
+// enqueues the copies of one or two sets, gamma_end waits for them and judges
+// them (after a refusal, with the stream idle again).
+template <typename R>
+int gamma_begin(ace_plan* P, const void* psi, int n, const void* psi2, int n2, cudaStream_t st) {
+    const size_t need = (size_t)(n + n2) * sizeof(cx<R>);
+    if (need > P->hg_cap) {
+        if (P->h_gamma) cudaFreeHost(P->h_gamma);
+        P->h_gamma = nullptr;
+        P->hg_cap = 0;
+        if (cudaMallocHost(&P->h_gamma, need) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(ACE_ERR_OOM, "pinned host allocation failed");
+        }
+        P->hg_cap = need;
+    }
+    if (!P->gamma_ev) ACE_CK(cudaEventCreateWithFlags(&P->gamma_ev, cudaEventDisableTiming));
+    cx<R>* h = (cx<R>*)P->h_gamma;
+    const size_t pitch = (size_t)P->npw * sizeof(cx<R>);
+    ACE_CK(cudaMemcpy2DAsync(h, sizeof(cx<R>), psi, pitch, sizeof(cx<R>), n, cudaMemcpyDeviceToHost, st));
+    if (n2 > 0)
+        ACE_CK(cudaMemcpy2DAsync(h + n, sizeof(cx<R>), psi2, pitch, sizeof(cx<R>), n2, cudaMemcpyDeviceToHost, st));
+    ACE_CK(cudaEventRecord(P->gamma_ev, st));
+    return ACE_OK;
+}
+
+template <typename R>
+int gamma_end(ace_plan* P, int n, int n2, cudaStream_t st) {
+    ACE_CK(cudaEventSynchronize(P->gamma_ev));
+    const cx<R>* h = (const cx<R>*)P->h_gamma;
+    for (int i = 0; i < n + n2; ++i)
+        if (std::fabs((double)h[i].im) > 1e-6) {
+            ACE_CK(cudaStreamSynchronize(st));
+            return fail(ACE_ERR_INVALID_ARG,
+                        "Im c(G=0) of vector " + std::to_string(i < n ? i : i - n) + " is not zero");
+        }
+    return ACE_OK;
+}
+
 template <typename R>
 int check_gamma(ace_plan* P, const void* psi, int n, cudaStream_t st) {
-    std::vector<cx<R>> c0(n);
-    ACE_CK(cudaMemcpy2DAsync(c0.data(), sizeof(cx<R>), psi, (size_t)P->npw * sizeof(cx<R>), sizeof(cx<R>), n,
-                             cudaMemcpyDeviceToHost, st));
-    ACE_CK(cudaStreamSynchronize(st));
-    for (int i = 0; i < n; ++i)
-        if (std::fabs((double)c0[i].im) > 1e-6)
-            return fail(ACE_ERR_INVALID_ARG, "Im c(G=0) of vector " + std::to_string(i) + " is not zero");
-    return ACE_OK;
+    ACE_TRY(gamma_begin<R>(P, psi, n, nullptr, 0, st));
+    return gamma_end<R>(P, n, 0, st);
 }
 
 // The quads go through the plan's pinned staging buffer (a captured copy
@@ -762,9 +799,13 @@ int upload_quads(ace_plan* P, const std::vector<Quad>& q, cudaStream_t st) {
 // validated for the Gamma point): phi(r), every listed pair's Poisson solve
 // with the exchange accumulation (Eq. 2-4), W -> W_G (into WG) and E_x over
 // the listed pairs (into the plan's pinned host slot).
+// check: the Gamma-point check of psi_G runs here (its copy behind the pair
+// list's preparation and the orbital transforms, before anything that outlives a
+// refused call is written).
 template <typename R>
 int pairs_enqueue(ace_plan* P, const void* psi_G, int n_occ, double alpha, const int32_t* rp, const int32_t* col,
-                  void* WG_out, cudaStream_t st) {
+                  void* WG_out, cudaStream_t st, bool check) {
+    if (check) ACE_TRY(gamma_begin<R>(P, psi_G, n_occ, nullptr, 0, st));
     std::vector<int> pa, pb;
     if (rp) {
         if (rp[0] != 0) return fail(ACE_ERR_INVALID_ARG, "pair_row_ptr[0] must be 0");
@@ -800,6 +841,7 @@ int pairs_enqueue(ace_plan* P, const void* psi_G, int n_occ, double alpha, const
     R* phi = (R*)P->d_phi;
     R* acc = (R*)P->d_acc;
     ACE_TRY(run_to_real<R>(P, psi, d_oq, n_orb_t, phi, st));
+    if (check) ACE_TRY(gamma_end<R>(P, n_occ, 0, st));
     ACE_CK(cudaMemsetAsync(acc, 0, (size_t)n_occ * P->N * sizeof(R), st));
     ACE_TRY(grow(&P->d_epart, &P->epart_cap, (size_t)std::max(n_pair_t, 1) * P->ntiles_last * 2));
     ACE_TRY(run_pairs<R>(P, phi, phi, acc, acc, 1, d_pq, n_pair_t, P->d_epart, st));
@@ -846,14 +888,13 @@ int finish_enqueue(ace_plan* P, const void* psi_G, int n_occ, const void* WG_in,
 // pinned host slots.
 template <typename R>
 int build_enqueue(ace_plan* P, const void* psi_G, int n_occ, double alpha, const int32_t* rp, const int32_t* col,
-                  void* xi, cudaStream_t st) {
-    ACE_TRY(pairs_enqueue<R>(P, psi_G, n_occ, alpha, rp, col, P->d_WG, st));
+                  void* xi, cudaStream_t st, bool check) {
+    ACE_TRY(pairs_enqueue<R>(P, psi_G, n_occ, alpha, rp, col, P->d_WG, st, check));
     return finish_enqueue<R>(P, psi_G, n_occ, P->d_WG, xi, st);
 }
 
 // Wait for an enqueued build and report its result.
 int build_finish(ace_plan* P, double* E_x, cudaStream_t st) {
-    ACE_CK(cudaStreamSynchronize(st));
     ACE_TRY(check_device_error(P, st));
     P->last_n_occ = P->pending_n_occ;
     if (E_x) *E_x = P->h_res->E;
@@ -864,9 +905,7 @@ int build_finish(ace_plan* P, double* E_x, cudaStream_t st) {
 template <typename R>
 int pairs_impl(ace_plan* P, const void* psi_G, int n_occ, double alpha, const int32_t* rp, const int32_t* col,
                void* WG, double* E_part, cudaStream_t st) {
-    ACE_TRY(check_gamma<R>(P, psi_G, n_occ, st));
-    ACE_TRY(pairs_enqueue<R>(P, psi_G, n_occ, alpha, rp, col, WG, st));
-    ACE_CK(cudaStreamSynchronize(st));
+    ACE_TRY(pairs_enqueue<R>(P, psi_G, n_occ, alpha, rp, col, WG, st, true));
     ACE_TRY(check_device_error(P, st));
     if (E_part) *E_part = P->h_res->E;
     return ACE_OK;
@@ -882,16 +921,14 @@ int finish_impl(ace_plan* P, const void* psi_G, int n_occ, const void* WG, void*
 template <typename R>
 int build_impl(ace_plan* P, const void* psi_G, int n_occ, double alpha, const int32_t* rp, const int32_t* col,
                void* xi, double* E_x, cudaStream_t st) {
-    ACE_TRY(check_gamma<R>(P, psi_G, n_occ, st));
-    ACE_TRY(build_enqueue<R>(P, psi_G, n_occ, alpha, rp, col, xi, st));
+    ACE_TRY(build_enqueue<R>(P, psi_G, n_occ, alpha, rp, col, xi, st, true));
     return build_finish(P, E_x, st);
 }
 
 template <typename R>
 int hfx_impl(ace_plan* P, const void* psi_occ, int n_occ, double alpha, const void* psi, int T, void* out,
              cudaStream_t st) {
-    ACE_TRY(check_gamma<R>(P, psi_occ, n_occ, st));
-    ACE_TRY(check_gamma<R>(P, psi, T, st));
+    ACE_TRY(gamma_begin<R>(P, psi_occ, n_occ, psi, T, st));
     std::vector<Quad> oq = orbital_quads(n_occ), tq = orbital_quads(T), q = oq;
     q.insert(q.end(), tq.begin(), tq.end());
     std::vector<int> pa, pb;
@@ -918,6 +955,7 @@ int hfx_impl(ace_plan* P, const void* psi_occ, int n_occ, double alpha, const vo
     R* phi = (R*)P->d_phi;
     ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi_occ, P->d_quads, no, phi, st));
     ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi, P->d_quads + no, nt, (R*)tphi, st));
+    ACE_TRY(gamma_end<R>(P, n_occ, T, st));
     ACE_CK(cudaMemsetAsync(P->d_tacc, 0, (size_t)T * P->N * sizeof(R), st));
     ACE_TRY(run_pairs<R>(P, (const R*)tphi, phi, (R*)P->d_tacc, nullptr, 0, P->d_quads + no + nt, np, nullptr, st));
     const double g = phi_gain<R>(P);
@@ -935,12 +973,13 @@ int hfx_impl(ace_plan* P, const void* psi_occ, int n_occ, double alpha, const vo
 template <typename R>
 int overlap_impl(ace_plan* P, const void* psi_G, int n, double rho_cut, int32_t* rp, int32_t* col, int* n_pairs,
                  double* S_out, cudaStream_t st) {
-    ACE_TRY(check_gamma<R>(P, psi_G, n, st));
+    ACE_TRY(gamma_begin<R>(P, psi_G, n, nullptr, 0, st));
     std::vector<Quad> oq = orbital_quads(n);
     ACE_TRY(upload_quads_eager(P, oq, st));
     ACE_TRY(grow(&P->d_S, &P->S_cap, (size_t)n * n));
     R* phi = (R*)P->d_phi;
     ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi_G, P->d_quads, (int)oq.size(), phi, st));
+    ACE_TRY(gamma_end<R>(P, n, 0, st));
     const long long K = P->N;
     const double g = phi_gain<R>(P);
     const double scale = P->omega / (double)P->N / (g * g);
@@ -970,7 +1009,6 @@ int overlap_impl(ace_plan* P, const void* psi_G, int n, double rho_cut, int32_t*
     mark(P, PH_IDLE, st);
     std::vector<double> S((size_t)n * n);
     ACE_CK(cudaMemcpyAsync(S.data(), P->d_S, S.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-    ACE_CK(cudaStreamSynchronize(st));
     ACE_TRY(check_device_error(P, st));
     int q = 0;
     rp[0] = 0;
@@ -1091,7 +1129,6 @@ int scdm_impl(ace_plan* P, const void* psi_G, int n, int preselect, void* phi_G,
         ACE_CK(cudaMemcpyAsync(pivots, grid_pts, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, st));
     }
     if (O) ACE_CK(cudaMemcpyAsync(O, X, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    ACE_CK(cudaStreamSynchronize(st));
     ACE_TRY(check_device_error(P, st));
     if (n_cand) *n_cand = (int)m;
     return ACE_OK;
@@ -1150,13 +1187,14 @@ int apply_energy_impl(ace_plan* P, const void* xi, int n_occ, const void* psi, i
     }
     mark(P, PH_IDLE, st);
     ACE_CK(cudaMemcpyAsync(&P->h_res->E, P->d_E, sizeof(double), cudaMemcpyDeviceToHost, st));
-    ACE_CK(cudaStreamSynchronize(st));
     ACE_TRY(check_device_error(P, st));
     *E = P->h_res->E;
     return ACE_OK;
 }
 
 void free_plan(ace_plan* P) {
+    if (P->gamma_ev) cudaEventDestroy(P->gamma_ev);
+    if (P->h_gamma) cudaFreeHost(P->h_gamma);
     if (P->h_res) cudaFreeHost(P->h_res);
     if (P->quads_ev) cudaEventSynchronize(P->quads_ev);
     if (P->h_quads) cudaFreeHost(P->h_quads);
@@ -1580,7 +1618,7 @@ int create_impl(ace_plan* P, const ace_opts* opts) {
     ACE_TRY(dalloc((void**)&P->d_in, P->npw * sizeof(int)));
     ACE_CK(cudaMemcpy(P->d_ip, ip.data(), P->npw * sizeof(int), cudaMemcpyHostToDevice));
     ACE_CK(cudaMemcpy(P->d_in, in.data(), P->npw * sizeof(int), cudaMemcpyHostToDevice));
-    P->sphere = sizeof(R) == 4 && P->fused_xy && generic_supported(P->n[0], P->n[1], P->n[2], 226 * 1024);
+    P->sphere = sizeof(R) == 4 && P->fused_xy && generic_supported(P->n[0], P->n[1], P->n[2]);
     if (P->sphere) {
         // pencil (plane position) -> its plane waves, +G and -G
         const int plane = P->n[1] * P->n[2], unit = sphere_unit(P->n[1], P->n[2]);
@@ -1719,8 +1757,8 @@ int ace_build_async(ace_plan* plan, const void* psi_G, int n_occ, double alpha, 
     cudaStream_t st = (cudaStream_t)stream;
     g_capture = capturing(st);
     const int rc = plan->prec == ACE_FP64
-                       ? build_enqueue<double>(plan, psi_G, n_occ, alpha, pair_row_ptr, pair_col, xi, st)
-                       : build_enqueue<float>(plan, psi_G, n_occ, alpha, pair_row_ptr, pair_col, xi, st);
+                       ? build_enqueue<double>(plan, psi_G, n_occ, alpha, pair_row_ptr, pair_col, xi, st, false)
+                       : build_enqueue<float>(plan, psi_G, n_occ, alpha, pair_row_ptr, pair_col, xi, st, false);
     g_capture = false;
     return rc;
 }
@@ -1886,8 +1924,8 @@ int ace_build_batched(ace_system* sys, int n_sys, void* stream) {
             break;
         }
         s.status = s.plan->prec == ACE_FP64
-                       ? build_enqueue<double>(s.plan, s.psi_G, s.n_occ, s.alpha, s.pair_row_ptr, s.pair_col, s.xi, ss[i])
-                       : build_enqueue<float>(s.plan, s.psi_G, s.n_occ, s.alpha, s.pair_row_ptr, s.pair_col, s.xi, ss[i]);
+                       ? build_enqueue<double>(s.plan, s.psi_G, s.n_occ, s.alpha, s.pair_row_ptr, s.pair_col, s.xi, ss[i], false)
+                       : build_enqueue<float>(s.plan, s.psi_G, s.n_occ, s.alpha, s.pair_row_ptr, s.pair_col, s.xi, ss[i], false);
         if (s.status != ACE_OK) rc = s.status;
         cudaEventRecord(done[i], ss[i]);
     }

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "fft_core.cuh"
 
 namespace ace {
@@ -185,6 +187,24 @@ inline bool stream_capturing(cudaStream_t st) {
     return cs != cudaStreamCaptureStatusNone;
 }
 
+// Shared-memory limit (and, with full_carveout, the whole L1 carveout) of a
+// kernel, set on its first launch on each device outside stream capture: the two
+// attribute calls cost some microseconds, as much as a small launch.  `done`: a
+// static of the launcher, one bit per device.
+inline cudaError_t kernel_limits(const void* kernel, int smem, bool full_carveout, std::atomic<unsigned long long>& done,
+                                 cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if ((done.load(std::memory_order_acquire) & bit) || stream_capturing(st)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess && full_carveout)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
 // compile-time cube passes (cube_*.cu), single precision
 cudaError_t cube_pass_launch(int n, const PassArgs& a, const PassShape& s, int pro, int epi, int mid, int sgn,
                              int batch, cudaStream_t st);
@@ -194,7 +214,7 @@ cudaError_t cube_pass_launch(int n, const PassArgs& a, const PassShape& s, int p
 // passes (PRO_PAIR / PRO_PACK2 with EPI_STORE; EPI_ACCUM / EPI_SPLIT), pencil
 // passes (mode -1 forward z, +1 inverse z, 0 forward z, times PassArgs::kern,
 // inverse z).
-bool generic_supported(int n0, int n1, int n2, size_t smem_limit);
+bool generic_supported(int n0, int n1, int n2);  // on the current device
 cudaError_t generic_plane_launch(const PassArgs& a, int pro, int epi, int batch, cudaStream_t st);
 cudaError_t generic_pencil_launch(const PassArgs& a, int mode, int batch, cudaStream_t st);
 

@@ -744,11 +744,16 @@ __global__ void __launch_bounds__(Shape::kMaxThreads, Shape::kMinBlocks) tile_pa
 template <typename Shape, typename R, int PRO, int EPI, int MID, int SGN>
 cudaError_t launch_one(const PassArgs& a, const PassShape& s, int batch, cudaStream_t st) {
     auto k = tile_pass<Shape, R, PRO, EPI, MID, SGN>;
-    if (s.smem > 48 * 1024 && !stream_capturing(st)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
-        if (e == cudaSuccess && Shape::kMinBlocks > 2)  // three plane blocks need the whole shared carveout
-            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
+    if (s.smem > 48 * 1024) {
+        if constexpr (Shape::kCube) {  // one tile size per kernel
+            static std::atomic<unsigned long long> done{0};
+            // three plane blocks need the whole shared carveout
+            cudaError_t e = kernel_limits((const void*)k, (int)s.smem, Shape::kMinBlocks > 2, done, st);
+            if (e != cudaSuccess) return e;
+        } else if (!stream_capturing(st)) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+            if (e != cudaSuccess) return e;
+        }
     }
     const int ntiles = (a.n0 / s.tz) * (a.n1 / s.ty) * (a.n2 / s.tx);
     dim3 grid(ntiles, batch);

@@ -445,10 +445,11 @@ __global__ void __launch_bounds__(Geo<N, F0, TPL>::NT, Geo<N, F0, TPL>::kMinBloc
                        a.e_part != nullptr ? a.e_part + ((long long)(a.t0 + t) * gridDim.x + z) * 2 : nullptr);
 }
 
-template <typename K>
-cudaError_t launch_plane(K k, size_t smem, int n, int nt, const PassArgs& a, int batch, cudaStream_t st) {
-    if (smem > 48 * 1024 && !stream_capturing(st)) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <void (*k)(PassArgs)>
+cudaError_t launch_plane(size_t smem, int n, int nt, const PassArgs& a, int batch, cudaStream_t st) {
+    if (smem > 48 * 1024) {
+        static std::atomic<unsigned long long> done{0};
+        cudaError_t e = kernel_limits((const void*)k, (int)smem, false, done, st);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)n, (unsigned)batch);
@@ -467,13 +468,13 @@ cudaError_t tplane_launch(int which, const PassArgs& a, int batch, cudaStream_t 
                                            // blocks of four threads per line ran P1 4% slower than three of two)
     using G = plane_detail::Geo<N, F0, TPL>;
     if (which == 2)
-        return plane_detail::launch_plane(plane_detail::pair_fwd<N, true, F0, TPL>, G::smem, N, G::NT, a, batch, st);
+        return plane_detail::launch_plane<plane_detail::pair_fwd<N, true, F0, TPL>>(G::smem, N, G::NT, a, batch, st);
     if constexpr (N % 8 != 0) {
         return cudaErrorInvalidValue;  // transposed planes: n % 8 == 0 only
     } else {
         if (which == 0)
-            return plane_detail::launch_plane(plane_detail::pair_fwd<N, false, F0, TPL>, G::smem, N, G::NT, a, batch, st);
-        return plane_detail::launch_plane(plane_detail::inv_accum<N, F0, TPL>, G::smem, N, G::NT, a, batch, st);
+            return plane_detail::launch_plane<plane_detail::pair_fwd<N, false, F0, TPL>>(G::smem, N, G::NT, a, batch, st);
+        return plane_detail::launch_plane<plane_detail::inv_accum<N, F0, TPL>>(G::smem, N, G::NT, a, batch, st);
     }
 }
 
