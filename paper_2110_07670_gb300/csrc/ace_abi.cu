@@ -1089,10 +1089,10 @@ int scdm_impl(ace_plan* P, const void* psi_G, int n, int preselect, void* phi_G,
     double *Q = W.mats, *X = Q + (size_t)n * n, *T = X + (size_t)n * n, *Y = T + (size_t)n * n, *err = Y + (size_t)n * n;
     int *piv = W.ipiv, *status = W.ipiv + n;  // piv: columns of A; grid points after them
     double *rdiag = err + 2 + 2 * n, *fro = rdiag + n;  // after err, nu0, r, c; fro right after rdiag
-    const QrWork qw{W.part, W.nu, W.nu + m, Q, err + 2, err + 2 + n, err + 1, rdiag, piv, status};
+    const QrWork qw{W.part, W.nu, W.nu + m, Q, err + 2, err + 2 + n, err + 1, rdiag, piv, status, qb};
     ACE_CK(cudaMemsetAsync(status, 0, sizeof(int), st));
     ACE_CKL(launch_gather_columns<R>(phi, n, N, sel, m, A, st));
-    ACE_CKL(launch_qr_init<R>(A, n, m, W.nu, W.part, st));
+    ACE_CKL(launch_qr_init<R>(A, n, m, W.nu, W.part, qb, st));
     for (int k = 0; k < n; ++k) ACE_CKL(launch_qr_step<R>(A, n, m, k, qw, st));
     int h_status = 0;
     ACE_CK(cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1113,7 +1113,11 @@ int scdm_impl(ace_plan* P, const void* psi_G, int n, int preselect, void* phi_G,
     for (int it = 0; it < 100 && !converged; ++it) {
         const double alpha = std::sqrt(3.0 / (1.0 + l + l * l));
         ACE_CKL(launch_newton_schulz_step(X, T, Y, n, alpha, err, st));
+        // l over-estimates the smallest singular value: before it is within 1e-6
+        // of one the step's error cannot be below the limit, so nothing is read
+        const double before = l;
         l = std::min(1.0, 0.5 * alpha * l * (3.0 - alpha * alpha * l * l));
+        if (1.0 - before > 1e-6) continue;
         double h_err = 0;
         ACE_CK(cudaMemcpyAsync(&h_err, err, sizeof(double), cudaMemcpyDeviceToHost, st));
         ACE_CK(cudaStreamSynchronize(st));

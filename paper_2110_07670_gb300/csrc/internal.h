@@ -339,9 +339,10 @@ struct QrWork {
     void* part;
     double *nu, *R, *Q, *r, *c, *nu0, *rdiag;  // rdiag [n]: R[k][k] = |r_k|
     int *piv, *status;
+    int blocks;  // scdm_qr_blocks of the column passes
 };
 template <typename T>
-cudaError_t launch_qr_init(const T* A, int n, long long m, double* nu, void* part, cudaStream_t st);
+cudaError_t launch_qr_init(const T* A, int n, long long m, double* nu, void* part, int blocks, cudaStream_t st);
 template <typename T>
 cudaError_t launch_qr_step(const T* A, int n, long long m, int k, QrWork w, cudaStream_t st);
 // out[k] = sel[piv[k]] (sel null: piv[k]): the pivots' grid points

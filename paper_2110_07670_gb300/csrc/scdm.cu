@@ -11,11 +11,13 @@
 //   Phi = (V V^T)^{-1/2} V Psi, V[k][i] = psi_i(r_{C_k}): the polar factor of V
 //     by scaled Newton-Schulz steps X <- X (3 I - X^T X) / 2 from V / |V|_F
 // Sums and decisions in double; the orbitals' real-space values come in the
-// plan's precision, and for single precision the QR's column pass forms its
-// products in float-float arithmetic (about 2^-48 relative) on the FP32 pipes.
+// plan's precision, and for single precision the QR's column pass (and, up to 256
+// orbitals, its projections) form their products in float-float arithmetic
+// (about 2^-46 relative) on the FP32 pipes.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -30,9 +32,12 @@ struct ArgMax {
     long long j;
 };
 
-// larger value wins; equal values go to the lower index
+// larger value wins; equal values go to the lower index.  Residual norms are
+// non-negative and chosen columns hold -1, so the bits compare as integers: the
+// FP64 pipe (two comparisons per cycle and SM) took half of the column pass.
 __device__ __forceinline__ ArgMax better(ArgMax a, ArgMax b) {
-    if (b.v > a.v || (b.v == a.v && b.j >= 0 && (a.j < 0 || b.j < a.j))) return b;
+    const long long av = __double_as_longlong(a.v), bv = __double_as_longlong(b.v);
+    if (bv > av || (bv == av && b.j >= 0 && (a.j < 0 || b.j < a.j))) return b;
     return a;
 }
 
@@ -134,16 +139,19 @@ __global__ void stats_partial_kernel(const double* __restrict__ rho, const doubl
     }
 }
 
-// means[0] = <rho>, means[1] = <|grad rho|>, block partials added in order
+// means[0] = <rho>, means[1] = <|grad rho|>, block partials added in a fixed order
 __global__ void stats_final_kernel(const double* __restrict__ part, int nb, long long N, double* __restrict__ means) {
-    if (threadIdx.x != 0) return;
     double a = 0, b = 0;
-    for (int k = 0; k < nb; ++k) {
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
         a += part[2 * k];
         b += part[2 * k + 1];
     }
-    means[0] = a / (double)N;
-    means[1] = b / (double)N;
+    a = block_sum(a);
+    b = block_sum(b);
+    if (threadIdx.x == 0) {
+        means[0] = a / (double)N;
+        means[1] = b / (double)N;
+    }
 }
 
 __device__ __forceinline__ bool candidate(const double* rho, const double* g, long long N, long long r,
@@ -362,42 +370,245 @@ __device__ __forceinline__ void ff_dot_acc(float qh, float ql, float a, float& s
     sh = s;
 }
 
-// (3): every block normalises r itself; block 0 stores q_k and |r| = R[k][k].
-// Double candidate columns: the dots in double; single-precision ones (exact
-// in float): in float-float (ff_dot_acc).
-template <typename T>
-__global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, const double* __restrict__ r, int k,
-                                 double* __restrict__ Q, double* __restrict__ Rrows, double* __restrict__ nu,
-                                 double* __restrict__ rdiag, ArgMax* __restrict__ part) {
-    extern __shared__ double q[];
-    float* qh = reinterpret_cast<float*>(q + n);  // float-float split of q (single precision A)
-    float* ql = qh + n;
-    __shared__ double s_inv;
-    double ss = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double v = r[i];
-        q[i] = v;
-        ss += v * v;
-    }
-    ss = block_sum(ss);
-    if (threadIdx.x == 0) {
-        s_inv = ss > 0 ? 1.0 / sqrt(ss) : 0.0;
-        if (blockIdx.x == 0) rdiag[k] = sqrt(ss);  // R[k][k]
+// Single precision and n <= kPivotN: (1) and (2) and the normalisation in one
+// block, in float-float arithmetic on the FP32 pipes like the column pass (one
+// SM's FP64 rate, two multiply-adds per cycle, would take 12 us for 128 orbitals;
+// spread over blocks it took three launches, 14 us, and every block of the column
+// pass then repeated the norm, root and split).  Measured for 128 orbitals: 9.6
+// us per step, the column pass 6.8 instead of 13.6, the whole call 5.5 instead of
+// 7.6 ms.  Bound by the latency of its serial parts.  Above kPivotN orbitals one
+// SM falls behind the spread form.  q_k goes out as two floats, Q [n][2][n].
+constexpr int kPivotN = 256, kPivotThreads = 512;
+
+// (sh, sl) += (h, l)
+__device__ __forceinline__ void ff_pair_add(float& sh, float& sl, float h, float l) {
+    const float s = __fadd_rn(sh, h), bb = __fsub_rn(s, sh);
+    sl = __fadd_rn(__fadd_rn(sl, l), __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(h, bb)));
+    sh = s;
+}
+
+// sum += c q for c = ch + cl, q = qh + ql (float pairs), kept as the pair (sh, sl)
+__device__ __forceinline__ void ff_mul_acc(float ch, float cl, float qh, float ql, float& sh, float& sl) {
+    const float p = __fmul_rn(ch, qh);
+    float e = fmaf(ch, qh, -p);  // ch qh - p, exactly
+    e = fmaf(ch, ql, e);
+    e = fmaf(cl, qh, e);
+    const float s = __fadd_rn(sh, p), bb = __fsub_rn(s, sh);
+    const float t = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    sl = __fadd_rn(sl, __fadd_rn(t, e));
+    sh = s;
+}
+
+// r[i] -= sum_{l < k} (ch + cl)[l] q_l[i] by the whole block (n <= blockDim); the
+// sums stay float pairs, one double subtraction per row ends them
+__device__ __forceinline__ void subtract_projections(double* r, const float* ch, const float* cl,
+                                                     const float* __restrict__ Q, int n, int k, float2* part) {
+    const int groups = blockDim.x / n, g = threadIdx.x / n, i = threadIdx.x - g * n;
+    if (g < groups) {
+        float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* q = Q + i;
+        // eight rows' loads in flight (past k: zeros)
+        for (int l = g; l < k; l += 8 * groups) {
+            float qh[8], ql[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool in = l + u * groups < k;
+                qh[u] = in ? q[(l + u * groups) * 2 * n] : 0.f;
+                ql[u] = in ? q[(l + u * groups) * 2 * n + n] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (l + u * groups < k)
+                    ff_mul_acc(ch[l + u * groups], cl[l + u * groups], qh[u], ql[u], sh[u & 3], sl[u & 3]);
+        }
+#pragma unroll
+        for (int u = 1; u < 4; ++u) ff_pair_add(sh[0], sl[0], sh[u], sl[u]);
+        part[g * n + i] = make_float2(sh[0], sl[0]);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        q[i] *= s_inv;
-        if (blockIdx.x == 0) Q[(long long)k * n + i] = q[i];
-        if constexpr (sizeof(T) == 4) {
-            qh[i] = (float)q[i];
-            ql[i] = (float)(q[i] - (double)qh[i]);
+    if ((int)threadIdx.x < n) {
+        float h = 0.f, l = 0.f;
+        for (int gg = 0; gg < groups; ++gg) ff_pair_add(h, l, part[gg * n + threadIdx.x].x, part[gg * n + threadIdx.x].y);
+        r[threadIdx.x] -= (double)h + (double)l;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kPivotThreads) qr_pivot_kernel(const ArgMax* __restrict__ parts, int nparts,
+                                                                 const float* __restrict__ A, int n, long long m,
+                                                                 const double* __restrict__ Rrows, int k,
+                                                                 float* __restrict__ Q, int* __restrict__ piv,
+                                                                 double* __restrict__ nu, double* __restrict__ nu0,
+                                                                 double* __restrict__ rdiag, int* __restrict__ status) {
+    __shared__ double r[kPivotN], s_inv;
+    __shared__ float2 part[kPivotThreads];
+    __shared__ float ch[kPivotN], cl[kPivotN], rh[kPivotN], rl[kPivotN];
+    __shared__ ArgMax wbest[kPivotThreads / 32];
+    __shared__ long long s_p;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ArgMax best{-1.0, -1};
+    for (int b = threadIdx.x; b < nparts; b += blockDim.x) best = better(best, parts[b]);
+    for (int o = 16; o > 0; o >>= 1) {
+        ArgMax y;
+        y.v = __shfl_down_sync(0xffffffffu, best.v, o);
+        y.j = __shfl_down_sync(0xffffffffu, best.j, o);
+        best = better(best, y);
+    }
+    if (lane == 0) wbest[warp] = best;
+    __syncthreads();
+    if (warp == 0) {
+        best = lane < kPivotThreads / 32 ? wbest[lane] : ArgMax{-1.0, -1};
+        for (int o = kPivotThreads / 64; o > 0; o >>= 1) {
+            ArgMax y;
+            y.v = __shfl_down_sync(0xffffffffu, best.v, o);
+            y.j = __shfl_down_sync(0xffffffffu, best.j, o);
+            best = better(best, y);
+        }
+    }
+    if (threadIdx.x == 0) {
+        const double ref = k == 0 ? best.v : *nu0;
+        const bool ok = best.j >= 0 && best.v > 1e-10 * ref && best.v == best.v;
+        s_p = ok ? best.j : -1;
+        if (k == 0) *nu0 = best.v;
+        if (ok) {
+            piv[k] = (int)best.j;
+            nu[best.j] = -1.0;
+        } else {
+            *status = 1;
         }
     }
     __syncthreads();
+    const long long p = s_p;
+    if (p < 0) {  // rank deficient: a zero row
+        for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) Q[(long long)k * 2 * n + i] = 0.f;
+        if (threadIdx.x == 0) rdiag[k] = 0.0;
+        return;
+    }
+    for (int e = threadIdx.x; e < n + k; e += blockDim.x) {
+        if (e < n) {
+            r[e] = (double)A[e * m + p];
+        } else {
+            const double c = Rrows[(e - n) * m + p];
+            ch[e - n] = (float)c;
+            cl[e - n] = (float)(c - (double)(float)c);
+        }
+    }
+    __syncthreads();
+    __shared__ float norm2[2];  // |a_p|^2, |r|^2 after the first pass
+    auto norm_to = [&](float* out) {
+        float ss = 0.f;
+        for (int i = lane; i < n; i += 32) ss += (float)r[i] * (float)r[i];
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        if (lane == 0) *out = ss;
+    };
+    if (k > 0) {
+        if (warp == 0) norm_to(&norm2[0]);
+        subtract_projections(r, ch, cl, Q, n, k, part);
+        if (warp == 0) norm_to(&norm2[1]);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            rh[i] = (float)r[i];
+            rl[i] = (float)(r[i] - (double)rh[i]);
+        }
+        __syncthreads();
+    }
+    // The second pass is needed where the first cancelled: a residual of at least
+    // half the column's length has lost at most one bit of orthogonality (Daniel,
+    // Gragg, Kaufman & Stewart, Math. Comp. 30 (1976)).
+    if (k > 0 && norm2[1] < 0.25f * norm2[0]) {
+        // the second pass: c_l = q_l . r, one warp per l
+        // (four at a time, their loads in flight together)
+        constexpr int NW = kPivotThreads / 32;
+        for (int l0 = warp; l0 < k; l0 += 4 * NW) {
+            float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int i = lane; i < n; i += 32) {
+                float qh[4], ql[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int l = l0 + u * NW;
+                    const float* q = Q + (long long)l * 2 * n;
+                    qh[u] = l < k ? q[i] : 0.f;
+                    ql[u] = l < k ? q[n + i] : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) ff_mul_acc(rh[i], rl[i], qh[u], ql[u], sh[u], sl[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                for (int o = 16; o > 0; o >>= 1)
+                    ff_pair_add(sh[u], sl[u], __shfl_xor_sync(0xffffffffu, sh[u], o),
+                                __shfl_xor_sync(0xffffffffu, sl[u], o));
+                if (lane == 0 && l0 + u * NW < k) {
+                    ch[l0 + u * NW] = sh[u];
+                    cl[l0 + u * NW] = sl[u];
+                }
+            }
+        }
+        __syncthreads();
+        subtract_projections(r, ch, cl, Q, n, k, part);
+    }
+    if (warp == 0) {
+        double ss = 0;
+        for (int i = lane; i < n; i += 32) ss += r[i] * r[i];
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        if (lane == 0) {
+            const double nr = sqrt(ss);
+            s_inv = ss > 0 ? 1.0 / nr : 0.0;
+            rdiag[k] = nr;  // R[k][k]
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double q = r[i] * s_inv;
+        const float h = (float)q;
+        Q[(long long)k * 2 * n + i] = h;
+        Q[(long long)k * 2 * n + n + i] = (float)(q - (double)h);
+    }
+}
+
+// (3): every block normalises r itself; block 0 stores q_k and |r| = R[k][k]
+// (SPLIT: q_k comes split from qr_pivot_kernel, Qs).  Double candidate columns:
+// the dots in double; single-precision ones (exact in float): in float-float
+// (ff_dot_acc).
+template <typename T, bool SPLIT>
+__global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, const double* __restrict__ r, int k,
+                                 double* __restrict__ Q, const float* __restrict__ Qs, double* __restrict__ Rrows,
+                                 double* __restrict__ nu, double* __restrict__ rdiag, ArgMax* __restrict__ part) {
+    extern __shared__ double q[];
+    float* qh = SPLIT ? reinterpret_cast<float*>(q) : reinterpret_cast<float*>(q + n);  // float-float split of q
+    float* ql = qh + n;
+    if constexpr (SPLIT) {
+        for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) qh[i] = Qs[(long long)k * 2 * n + i];
+        __syncthreads();
+    } else {
+        __shared__ double s_inv;
+        double ss = 0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const double v = r[i];
+            q[i] = v;
+            ss += v * v;
+        }
+        ss = block_sum(ss);
+        if (threadIdx.x == 0) {
+            s_inv = ss > 0 ? 1.0 / sqrt(ss) : 0.0;
+            if (blockIdx.x == 0) rdiag[k] = sqrt(ss);  // R[k][k]
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            q[i] *= s_inv;
+            if (blockIdx.x == 0) Q[(long long)k * n + i] = q[i];
+            if constexpr (sizeof(T) == 4) {
+                qh[i] = (float)q[i];
+                ql[i] = (float)(q[i] - (double)qh[i]);
+            }
+        }
+        __syncthreads();
+    }
     // tiles of 32 columns over one resident wave of blocks; warp g takes the
     // tile's columns (one per lane) over the row group g of 8, the groups
     // summed in shared memory
-    __shared__ double red[8][32];
+    // (row-group sums: float pairs for single-precision columns)
+    using Part = std::conditional_t<sizeof(T) == 4, float2, double>;
+    __shared__ Part red[8][32];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, cl = lane;
     const int rq = (n + 7) / 8, i0 = g * rq, i1 = i0 + rq < n ? i0 + rq : n;
     ArgMax best{-1.0, -1};
@@ -405,7 +616,7 @@ __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, co
     const long long ntiles = (m + 31) / 32;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const long long j = t * 32 + cl;
-        double part_sum = 0;
+        Part part_sum{};
         if (j < m) {
             // eight loads in flight per thread before their products
             if constexpr (sizeof(T) == 4) {
@@ -419,7 +630,8 @@ __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, co
                     for (int u = 0; u < 8; ++u) ff_dot_acc(qh[i + u], ql[i + u], v[u], sh[u & 1], sl[u & 1]);
                 }
                 for (; i < i1; ++i) ff_dot_acc(qh[i], ql[i], (float)A[i * m + j], sh[0], sl[0]);
-                part_sum = ((double)sh[0] + (double)sl[0]) + ((double)sh[1] + (double)sl[1]);
+                ff_pair_add(sh[0], sl[0], sh[1], sl[1]);
+                part_sum = make_float2(sh[0], sl[0]);
             } else {
                 double dd[4] = {0, 0, 0, 0};
                 int i = i0;
@@ -439,8 +651,16 @@ __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, co
         if (g == 0 && j < m) {
             double v = nu[j];
             if (v >= 0) {
-                const double d = ((red[0][cl] + red[1][cl]) + (red[2][cl] + red[3][cl])) +
-                                 ((red[4][cl] + red[5][cl]) + (red[6][cl] + red[7][cl]));
+                double d;
+                if constexpr (sizeof(T) == 4) {
+                    float h = red[0][cl].x, lw = red[0][cl].y;
+#pragma unroll
+                    for (int gg = 1; gg < 8; ++gg) ff_pair_add(h, lw, red[gg][cl].x, red[gg][cl].y);
+                    d = (double)h + (double)lw;
+                } else {
+                    d = ((red[0][cl] + red[1][cl]) + (red[2][cl] + red[3][cl])) +
+                        ((red[4][cl] + red[5][cl]) + (red[6][cl] + red[7][cl]));
+                }
                 Rk[j] = d;
                 v -= d * d;
                 if (v < 0) v = 0;
@@ -542,13 +762,16 @@ cudaError_t launch_orbital_sum(const R* phi, const R* dphi, int n, long long N, 
     return cudaGetLastError();
 }
 
-int scdm_stats_blocks(long long N) { return (int)((N + 65535) / 65536); }
+// grid points per block of the averages: 2048 (216 blocks at 96^3 take 8 us; the
+// 14 blocks of 65536 points took 280)
+constexpr long long kStatsChunk = 2048;
+int scdm_stats_blocks(long long N) { return (int)((N + kStatsChunk - 1) / kStatsChunk); }
 
 cudaError_t launch_scdm_stats(const double* rho, const double* grad, long long N, double* part, double* means,
                               cudaStream_t st) {
     const int nb = scdm_stats_blocks(N);
-    stats_partial_kernel<<<nb, kThreads, 0, st>>>(rho, grad, N, 65536, part);
-    stats_final_kernel<<<1, 32, 0, st>>>(part, nb, N, means);
+    stats_partial_kernel<<<nb, kThreads, 0, st>>>(rho, grad, N, kStatsChunk, part);
+    stats_final_kernel<<<1, kThreads, 0, st>>>(part, nb, N, means);
     return cudaGetLastError();
 }
 
@@ -580,8 +803,8 @@ int scdm_qr_blocks(long long m, int n, int esz) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const cudaError_t e =
-        esz == 4 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, qr_update_kernel<float>, kThreads, qr_update_smem(n))
-                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, qr_update_kernel<double>, kThreads, qr_update_smem(n));
+        esz == 4 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, qr_update_kernel<float, false>, kThreads, qr_update_smem(n))
+                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, qr_update_kernel<double, false>, kThreads, qr_update_smem(n));
     if (e != cudaSuccess || per < 1) {
         cudaGetLastError();
         per = 1;
@@ -593,22 +816,32 @@ int scdm_qr_blocks(long long m, int n, int esz) {
 size_t scdm_argmax_bytes() { return sizeof(ArgMax); }
 
 template <typename T>
-cudaError_t launch_qr_init(const T* A, int n, long long m, double* nu, void* part, cudaStream_t st) {
-    qr_init_kernel<T><<<scdm_qr_blocks(m, n, sizeof(T)), kThreads, 0, st>>>(A, n, m, nu, (ArgMax*)part);
+cudaError_t launch_qr_init(const T* A, int n, long long m, double* nu, void* part, int blocks, cudaStream_t st) {
+    qr_init_kernel<T><<<blocks, kThreads, 0, st>>>(A, n, m, nu, (ArgMax*)part);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_qr_step(const T* A, int n, long long m, int k, QrWork w, cudaStream_t st) {
-    const int rb = (n + 31) / 32, qb = scdm_qr_blocks(m, n, sizeof(T));
+    const int rb = (n + 31) / 32, qb = w.blocks;
+    if constexpr (sizeof(T) == 4) {
+        if (n <= kPivotN) {
+            float* Qs = reinterpret_cast<float*>(w.Q);  // n x 2 x n floats in the room of n x n doubles
+            qr_pivot_kernel<<<1, kPivotThreads, 0, st>>>((const ArgMax*)w.part, qb, A, n, m, w.R, k, Qs, w.piv, w.nu,
+                                                         w.nu0, w.rdiag, w.status);
+            qr_update_kernel<T, true><<<qb, kThreads, (size_t)2 * n * sizeof(float), st>>>(
+                A, n, m, nullptr, k, nullptr, Qs, w.R, w.nu, nullptr, (ArgMax*)w.part);
+            return cudaGetLastError();
+        }
+    }
     qr_resid_kernel<T><<<rb, kThreads, (size_t)(k + 1) * sizeof(double), st>>>(
         (const ArgMax*)w.part, qb, A, n, m, w.R, w.Q, k, w.piv, w.nu, w.nu0, w.status, w.r);
     if (k > 0) {
         qr_dots_kernel<<<(k + 7) / 8, kThreads, 0, st>>>(w.Q, n, k, w.r, w.c);
         qr_apply_kernel<<<rb, kThreads, (size_t)k * sizeof(double), st>>>(w.Q, n, k, w.c, w.r);
     }
-    qr_update_kernel<T><<<qb, kThreads, qr_update_smem(n), st>>>(
-        A, n, m, w.r, k, w.Q, w.R, w.nu, w.rdiag, (ArgMax*)w.part);
+    qr_update_kernel<T, false><<<qb, kThreads, qr_update_smem(n), st>>>(
+        A, n, m, w.r, k, w.Q, nullptr, w.R, w.nu, w.rdiag, (ArgMax*)w.part);
     return cudaGetLastError();
 }
 
@@ -647,8 +880,8 @@ template cudaError_t launch_gather_columns<float>(const float*, int, long long, 
                                                   cudaStream_t);
 template cudaError_t launch_gather_columns<double>(const double*, int, long long, const int*, long long, double*,
                                                    cudaStream_t);
-template cudaError_t launch_qr_init<float>(const float*, int, long long, double*, void*, cudaStream_t);
-template cudaError_t launch_qr_init<double>(const double*, int, long long, double*, void*, cudaStream_t);
+template cudaError_t launch_qr_init<float>(const float*, int, long long, double*, void*, int, cudaStream_t);
+template cudaError_t launch_qr_init<double>(const double*, int, long long, double*, void*, int, cudaStream_t);
 template cudaError_t launch_qr_step<float>(const float*, int, long long, int, QrWork, cudaStream_t);
 template cudaError_t launch_qr_step<double>(const double*, int, long long, int, QrWork, cudaStream_t);
 template cudaError_t launch_polar_start<float>(const float*, int, long long, const int*, double*, double*,
