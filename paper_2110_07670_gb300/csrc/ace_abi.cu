@@ -1272,7 +1272,7 @@ int choose_pair_variant(ace_plan* P, const ace_opts* opts) {
                     "pair_variant 2 needs a single-precision n^3 plan with n in {32, 80, 96, 120, 160}");
     if (req == 3 && !p_ok)
         return fail(ACE_ERR_INVALID_ARG, "pair_variant 3 needs a single-precision n^3 plan with n in {32, 80, 96, 160}");
-    if (req == 4 && !h_ok)
+    if (req == 4 && !(h_ok && hybrid_on_request(P->n[0])))
         return fail(ACE_ERR_INVALID_ARG,
                     "pair_variant 4 needs a single-precision n^3 plan with n in {32, 60, 80, 90, 96, 100, 108, 120, 160}");
     if (req > 0) {

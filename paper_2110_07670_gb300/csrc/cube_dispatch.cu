@@ -12,6 +12,15 @@ namespace pass_detail {
     extern template cudaError_t dispatch_cube<N>(const PassArgs&, const PassShape&, int, int, int, int, int, \
                                                  cudaStream_t);
 ACE_CUBE_DECL(32)
+ACE_CUBE_DECL(36)
+ACE_CUBE_DECL(40)
+ACE_CUBE_DECL(48)
+ACE_CUBE_DECL(50)
+ACE_CUBE_DECL(54)
+ACE_CUBE_DECL(64)
+ACE_CUBE_DECL(72)
+ACE_CUBE_DECL(128)
+ACE_CUBE_DECL(144)
 ACE_CUBE_DECL(60)
 ACE_CUBE_DECL(80)
 ACE_CUBE_DECL(90)
@@ -48,6 +57,15 @@ constexpr int alt_key(int n, int r0) { return n * 32 + r0; }
 
 #define ACE_ZLINE_DECL(N) extern template cudaError_t zline_launch<N>(const PassArgs&, int, cudaStream_t);
 ACE_ZLINE_DECL(32)
+ACE_ZLINE_DECL(36)
+ACE_ZLINE_DECL(40)
+ACE_ZLINE_DECL(48)
+ACE_ZLINE_DECL(50)
+ACE_ZLINE_DECL(54)
+ACE_ZLINE_DECL(64)
+ACE_ZLINE_DECL(72)
+ACE_ZLINE_DECL(128)
+ACE_ZLINE_DECL(144)
 ACE_ZLINE_DECL(60)
 ACE_ZLINE_DECL(80)
 ACE_ZLINE_DECL(90)
@@ -70,6 +88,15 @@ cudaError_t zline_coulomb_launch(int n, const PassArgs& a, int batch, cudaStream
     }
     switch (n) {
         case 32: return zline_launch<32>(a, batch, st);
+        case 36: return zline_launch<36>(a, batch, st);
+        case 40: return zline_launch<40>(a, batch, st);
+        case 48: return zline_launch<48>(a, batch, st);
+        case 50: return zline_launch<50>(a, batch, st);
+        case 54: return zline_launch<54>(a, batch, st);
+        case 64: return zline_launch<64>(a, batch, st);
+        case 72: return zline_launch<72>(a, batch, st);
+        case 128: return zline_launch<128>(a, batch, st);
+        case 144: return zline_launch<144>(a, batch, st);
         case 60: return zline_launch<60>(a, batch, st);
         case 80: return zline_launch<80>(a, batch, st);
         case 90: return zline_launch<90>(a, batch, st);
@@ -84,6 +111,15 @@ cudaError_t zline_coulomb_launch(int n, const PassArgs& a, int batch, cudaStream
 
 #define ACE_TPLANE_DECL(N) extern template cudaError_t tplane_launch<N>(int, const PassArgs&, int, cudaStream_t);
 ACE_TPLANE_DECL(32)
+ACE_TPLANE_DECL(36)
+ACE_TPLANE_DECL(40)
+ACE_TPLANE_DECL(48)
+ACE_TPLANE_DECL(50)
+ACE_TPLANE_DECL(54)
+ACE_TPLANE_DECL(64)
+ACE_TPLANE_DECL(72)
+ACE_TPLANE_DECL(128)
+ACE_TPLANE_DECL(144)
 ACE_TPLANE_DECL(60)
 ACE_TPLANE_DECL(80)
 ACE_TPLANE_DECL(90)
@@ -106,6 +142,15 @@ cudaError_t tplane_pair_launch(int n, int which, const PassArgs& a, int batch, c
     }
     switch (n) {
         case 32: return tplane_launch<32>(which, a, batch, st);
+        case 36: return tplane_launch<36>(which, a, batch, st);
+        case 40: return tplane_launch<40>(which, a, batch, st);
+        case 48: return tplane_launch<48>(which, a, batch, st);
+        case 50: return tplane_launch<50>(which, a, batch, st);
+        case 54: return tplane_launch<54>(which, a, batch, st);
+        case 64: return tplane_launch<64>(which, a, batch, st);
+        case 72: return tplane_launch<72>(which, a, batch, st);
+        case 128: return tplane_launch<128>(which, a, batch, st);
+        case 144: return tplane_launch<144>(which, a, batch, st);
         case 60: return tplane_launch<60>(which, a, batch, st);
         case 80: return tplane_launch<80>(which, a, batch, st);
         case 90: return tplane_launch<90>(which, a, batch, st);
@@ -171,6 +216,15 @@ cudaError_t cube_pass_launch(int n, const PassArgs& a, const PassShape& s, int p
     }
     switch (n) {
         case 32: return dispatch_cube<32>(a, s, pro, epi, mid, sgn, batch, st);
+        case 36: return dispatch_cube<36>(a, s, pro, epi, mid, sgn, batch, st);
+        case 40: return dispatch_cube<40>(a, s, pro, epi, mid, sgn, batch, st);
+        case 48: return dispatch_cube<48>(a, s, pro, epi, mid, sgn, batch, st);
+        case 50: return dispatch_cube<50>(a, s, pro, epi, mid, sgn, batch, st);
+        case 54: return dispatch_cube<54>(a, s, pro, epi, mid, sgn, batch, st);
+        case 64: return dispatch_cube<64>(a, s, pro, epi, mid, sgn, batch, st);
+        case 72: return dispatch_cube<72>(a, s, pro, epi, mid, sgn, batch, st);
+        case 128: return dispatch_cube<128>(a, s, pro, epi, mid, sgn, batch, st);
+        case 144: return dispatch_cube<144>(a, s, pro, epi, mid, sgn, batch, st);
         case 60: return dispatch_cube<60>(a, s, pro, epi, mid, sgn, batch, st);
         case 80: return dispatch_cube<80>(a, s, pro, epi, mid, sgn, batch, st);
         case 90: return dispatch_cube<90>(a, s, pro, epi, mid, sgn, batch, st);

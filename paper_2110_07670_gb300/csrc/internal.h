@@ -80,6 +80,12 @@ struct PassShape {
 // N^3 boxes with compile-time pass kernels, and their tile geometry (shared by
 // the host planner and the kernel instantiations).
 constexpr bool cube_supported(int n) {
+    return n == 32 || n == 36 || n == 40 || n == 48 || n == 50 || n == 54 || n == 60 || n == 64 || n == 72 || n == 80 ||
+           n == 90 || n == 96 || n == 100 || n == 108 || n == 120 || n == 128 || n == 144 || n == 160;
+}
+// The boxes on which ace_opts.pair_variant 4 can be asked for; on the other
+// cubes the automatic choice may still be it.
+constexpr bool hybrid_on_request(int n) {
     return n == 32 || n == 60 || n == 80 || n == 90 || n == 96 || n == 100 || n == 108 || n == 120 || n == 160;
 }
 // threads of a plane block: the butterfly counts of both stages divide evenly
@@ -134,8 +140,8 @@ inline int pair_radix_alternatives(int n, int* r0) {
     }
 }
 // plane passes with transposed spectrum planes (plane.cuh), N^3 boxes with
-// N % 8 == 0: which = 0 pair product + forward, 1 inverse + exchange accumulation
-constexpr bool tplane_supported(int n) { return n % 8 == 0; }
+// n in {32, 80, 96, 120, 160}: which = 0 pair product + forward, 1 inverse + exchange accumulation
+constexpr bool tplane_supported(int n) { return n == 32 || n == 80 || n == 96 || n == 120 || n == 160; }
 // ... and as one persistent kernel (its pencil groups: 16 per warp, N / 16 warps)
 constexpr bool pipeline_supported(int n) { return n % 16 == 0; }
 cudaError_t tplane_pair_launch(int n, int which, const PassArgs& a, int batch, cudaStream_t st);

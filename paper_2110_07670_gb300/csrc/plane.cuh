@@ -469,8 +469,8 @@ cudaError_t tplane_launch(int which, const PassArgs& a, int batch, cudaStream_t 
     using G = plane_detail::Geo<N, F0, TPL>;
     if (which == 2)
         return plane_detail::launch_plane<plane_detail::pair_fwd<N, true, F0, TPL>>(G::smem, N, G::NT, a, batch, st);
-    if constexpr (N % 8 != 0) {
-        return cudaErrorInvalidValue;  // transposed planes: n % 8 == 0 only
+    if constexpr (!tplane_supported(N)) {
+        return cudaErrorInvalidValue;  // no transposed planes
     } else {
         if (which == 0)
             return plane_detail::launch_plane<plane_detail::pair_fwd<N, false, F0, TPL>>(G::smem, N, G::NT, a, batch, st);
