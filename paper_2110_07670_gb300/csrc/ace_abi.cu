@@ -116,6 +116,7 @@ struct ace_plan {
     bool zline = false;        // per-pencil Coulomb pass (zline.cuh) with the kernel table d_kern
     float* d_kern = nullptr;   // 4 pi / |G|^2 / N in the tile passes' spectrum layout (zline only)
     float* d_kern_t = nullptr; // the same for transposed planes (n % 8 == 0 cubes)
+    float* d_kern_p = nullptr; // the same for padded natural planes (variant 4)
     double coul_rc = 0;        // Coulomb cutoff radius (0: 4 pi / |G|^2 with G = 0 dropped)
     int coul_g0 = 0;           // 1: the bare kernel keeps K(0) = 4 pi chi (auxiliary function)
     double coul_k0 = 0;        // that K(0)
@@ -133,7 +134,7 @@ struct ace_plan {
         size_t c_dpsi = 0, c_dens = 0, c_isel = 0, c_A = 0, c_nu = 0, c_part = 0, c_mats = 0, c_ipiv = 0;
     } scdm;
     int variant = 1;           // pair passes: 1 tile, 2 transposed planes, 3 persistent pipeline, 4 hybrid
-    bool hybrid = false;       // variant 4: plane-kernel P1 in the tile layout, then the tile P2 / P3
+    bool hybrid = false;       // variant 4: plane kernels with padded natural planes
     bool half = false;         // variant 5: P1 / P3 on clusters of two half-plane blocks (halfplane.cuh)
     float tune_ms[6] = {0, 0, 0, 0, 0, 0};  // autotune: tile x1 stream, tile x2, planes x2, pipeline, hybrid x2,
                                           // half planes x2
@@ -479,7 +480,7 @@ int pair_batch(ace_plan* P, PassArgs& a, int nb, cudaStream_t st, int lane) {
         mark(P, PH_PCOUL, st, lane);
         ACE_CKL(zline_coulomb_launch(P->n[0], a, nb, st));
         mark(P, PH_PINV, st, lane);
-        ACE_CKL(launch_pass<R>(a, P->s_xy, PRO_LOAD, EPI_ACCUM, MID_NONE, +1, nb, st));
+        ACE_CKL(tplane_pair_launch(P->n[0], 3, a, nb, st));
     } else if (P->fused_xy) {
         ACE_CKL(launch_pass<R>(a, P->s_xy, PRO_PAIR, EPI_STORE, MID_NONE, -1, nb, st));
         mark(P, PH_PCOUL, st, lane);
@@ -501,6 +502,9 @@ int pair_batch(ace_plan* P, PassArgs& a, int nb, cudaStream_t st, int lane) {
     return ACE_OK;
 }
 
+// Elements of a spectrum of padded natural planes (cube plans).
+long long natural_box(const ace_plan* P) { return (long long)P->n[0] * plane_stride(P->n[0]); }
+
 // Pair Poisson solves with fused exchange accumulation (Eq. 2-4).  With
 // pair_streams > 1 the transforms go in sub-batches round-robin over that many
 // streams forked from st (each with its own spectrum slots), so one
@@ -519,6 +523,11 @@ int run_pairs(ace_plan* P, const R* fl, const R* fr, R* accl, R* accr, int symme
     a.quads = dq;
     a.e_part = e_part;
     a.r0 = P->pair_r0;  // the spectrum tables were made for this plan
+    if (P->hybrid) {
+        a.natural = 1;
+        a.kern = P->d_kern_p;
+        a.src_tstride = a.dst_tstride = natural_box(P);
+    }
     if (P->fused && ntrans > 0) {
         // one persistent kernel over every transform (pipeline.cuh)
         ACE_TRY(grow(&P->d_pipe, &P->pipe_cap, (size_t)3 * ntrans + 2));
@@ -564,7 +573,7 @@ int run_pairs(ace_plan* P, const R* fl, const R* fr, R* accl, R* accr, int symme
         const int slot = k % S;
         PassArgs a2 = a;
         a2.t0 = t0;
-        a2.src = a2.dst = (cx<R>*)P->d_spec + (size_t)slot * b * P->N;
+        a2.src = a2.dst = (cx<R>*)P->d_spec + (size_t)slot * b * a.src_tstride;
         ACE_TRY(pair_batch<R>(P, a2, std::min(b, ntrans - t0), P->aux[slot], slot + 1));
     }
     for (int j = 0; j < S; ++j) {
@@ -1210,7 +1219,7 @@ void free_plan(ace_plan* P) {
     if (P->fork_ev) cudaEventDestroy(P->fork_ev);
     void* ptrs[] = {P->d_ip, P->d_in, P->d_sphere, P->d_tw[0], P->d_tw[1], P->d_tw[2], P->d_freq[0], P->d_freq[1], P->d_freq[2], P->d_phi, P->d_acc, P->d_spec,
                     P->d_WG, P->d_M, P->d_S, P->d_L, P->d_Linv, P->d_chol, P->d_E, P->d_status, P->d_err, P->d_part, P->d_quads,
-                    P->d_epart, P->d_tphi, P->d_tacc, P->d_C, P->d_kern, P->d_kern_t, P->d_kern_r, P->d_pipe, P->d_csplit, P->d_ximg,
+                    P->d_epart, P->d_tphi, P->d_tacc, P->d_C, P->d_kern, P->d_kern_t, P->d_kern_p, P->d_kern_r, P->d_pipe, P->d_csplit, P->d_ximg,
                     P->scdm.gv, P->scdm.dpsi, P->scdm.dens, P->scdm.isel, P->scdm.A, P->scdm.nu,
                     P->scdm.part, P->scdm.mats, P->scdm.ipiv};
     for (void* p : ptrs)
@@ -1515,7 +1524,8 @@ int pair_tables(ace_plan* P, int r0) {
     const int n0 = P->n[0], n1 = P->n[1], n2 = P->n[2];
     const bool with_t = P->zline && tplane_supported(n0);
     const bool swz_i = P->s_z.cube && cube_swizzle(n2);  // x slots of the tile passes' Coulomb stage
-    std::vector<float> kern(tab ? (size_t)P->N : 0), kern_t(with_t ? (size_t)P->N : 0);
+    std::vector<float> kern(tab ? (size_t)P->N : 0), kern_t(with_t ? (size_t)P->N : 0),
+        kern_p(P->zline ? (size_t)natural_box(P) : 0);
     std::vector<R> kern_r(inline_tab ? (size_t)P->N : 0);
     auto fold = [](int k, int n) { return k < n - n / 2 ? k : k - n; };
     auto g2_at = [&](int z, int y, int xp) {
@@ -1538,14 +1548,21 @@ int pair_tables(ace_plan* P, int r0) {
     for (int z = 0; z < n0; ++z)
         for (int y = 0; y < n1; ++y)
             for (int xs = 0; xs < n2; ++xs) {
-                const size_t e = ((size_t)z * n1 + y) * n2 + xs;
-                if (tab) kern[e] = (float)k(g2_at(z, y, swz ? plane_swizzle(xs, y, n2) : xs));
-                if (with_t) kern_t[((size_t)z * n2 + xs) * n1 + y] = (float)k(g2_at(z, y, xs));  // plane [x][y]
-                if (inline_tab) kern_r[e] = (R)k(g2_at(z, y, swz_i ? plane_swizzle(xs, y, n2) : xs));
+                // xs: position; its slot in a swizzled row is an involution of it
+                const size_t row = (size_t)z * n1 + y;
+                const double kv = k(g2_at(z, y, xs));
+                if (tab) kern[row * n2 + (swz ? plane_swizzle(xs, y, n2) : xs)] = (float)kv;
+                if (with_t) kern_t[((size_t)z * n2 + xs) * n1 + y] = (float)kv;  // plane [x][y]
+                if (P->zline) kern_p[(size_t)z * plane_stride(n0) + plane_row(n0, y) + xs] = (float)kv;  // (pads 0)
+                if (inline_tab) kern_r[row * n2 + (swz_i ? plane_swizzle(xs, y, n2) : xs)] = (R)kv;
             }
     if (with_t) {
         if (!P->d_kern_t) ACE_TRY(dalloc((void**)&P->d_kern_t, kern_t.size() * sizeof(float)));
         ACE_CK(cudaMemcpy(P->d_kern_t, kern_t.data(), kern_t.size() * sizeof(float), cudaMemcpyHostToDevice));
+    }
+    if (P->zline) {
+        if (!P->d_kern_p) ACE_TRY(dalloc((void**)&P->d_kern_p, kern_p.size() * sizeof(float)));
+        ACE_CK(cudaMemcpy(P->d_kern_p, kern_p.data(), kern_p.size() * sizeof(float), cudaMemcpyHostToDevice));
     }
     if (tab) {
         if (!P->d_kern) ACE_TRY(dalloc((void**)&P->d_kern, kern.size() * sizeof(float)));
@@ -1662,7 +1679,7 @@ int create_impl(ace_plan* P, const ace_opts* opts) {
     const size_t N = (size_t)P->N;
     ACE_TRY(dalloc(&P->d_phi, (size_t)P->n_occ_max * N * sizeof(R)));
     ACE_TRY(dalloc(&P->d_acc, (size_t)P->n_occ_max * N * sizeof(R)));
-    ACE_TRY(dalloc(&P->d_spec, (size_t)P->batch * N * sizeof(cx<R>)));
+    ACE_TRY(dalloc(&P->d_spec, (size_t)P->batch * (size_t)(P->zline ? natural_box(P) : N) * sizeof(cx<R>)));
     ACE_TRY(dalloc(&P->d_WG, (size_t)P->n_occ_max * P->npw * sizeof(cx<R>)));
     const size_t nn = (size_t)P->n_occ_max * P->n_occ_max;
     ACE_TRY(dalloc((void**)&P->d_M, nn * sizeof(double)));

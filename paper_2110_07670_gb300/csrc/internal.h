@@ -66,6 +66,7 @@ struct PassArgs {
     const void* kern;    // per-pencil Coulomb pass: 4 pi / |G|^2 / N in spectrum layout, [n0][n1][n2] float
     int kern_inline;     // 1: the tile passes' Coulomb stage reads K(G) / N from kern ([n0][n1][n2], type R,
                          // by x slot) instead of forming 4 pi / |G|^2 (cut-off interaction; double precision)
+    int natural;         // per-pencil Coulomb pass: 1: spectrum and kern in padded natural planes (plane_row)
     int r0;              // compile-time cube kernels: first radix of every axis (0: make_axis_plan's plan);
                          // nonzero only for the pair passes, with freq and kern made for that plan
 };
@@ -139,8 +140,26 @@ inline int pair_radix_alternatives(int n, int* r0) {
         default: return 0;
     }
 }
+// Natural planes of the plane passes (plane.cuh), in shared memory and in the
+// hybrid variant's spectrum: rows of n + 1 elements, an odd pitch that spreads
+// a column over the banks.  Where that leaves one block per SM and half the
+// padding fits two (n = 120: 2 x (115,712 + 1,024) bytes are all of 228 KB),
+// every second row is one element longer instead: with n = 8 (mod 16), 16
+// consecutive rows still start on 16 bank pairs.  (38 transforms of 120^3, one
+// block of 480 threads -> two of 384: forward plane pass 322 -> 269 us, inverse
+// 449 -> 366.)
+constexpr int plane_blocks(int bytes) { return 228 * 1024 / ((bytes + 127) / 128 * 128 + 1024); }
+constexpr bool plane_half_pad(int n) {
+    return n % 16 == 8 && plane_blocks((n * (n + 1) + n) * 8 + 16) == 1 && plane_blocks((n * n + n / 2) * 8 + 16) == 2;
+}
+constexpr int plane_elems(int n) { return n * n + (plane_half_pad(n) ? n / 2 : n); }
+// plane to plane in the spectrum: whole 128-byte lines
+constexpr int plane_stride(int n) { return (plane_elems(n) + 15) / 16 * 16; }
+__host__ __device__ constexpr int plane_row(int n, int y) { return n * y + (plane_half_pad(n) ? y >> 1 : y); }
+static_assert(plane_half_pad(120) && plane_row(120, 119) + 120 <= plane_elems(120), "the last row ends in the plane");
 // plane passes with transposed spectrum planes (plane.cuh), N^3 boxes with
-// n in {32, 80, 96, 120, 160}: which = 0 pair product + forward, 1 inverse + exchange accumulation
+// n in {32, 80, 96, 120, 160}: which = 0 pair product + forward, 1 inverse + exchange accumulation;
+// which = 2, 3: the same with natural planes (plane_row), on every cube
 constexpr bool tplane_supported(int n) { return n == 32 || n == 80 || n == 96 || n == 120 || n == 160; }
 // ... and as one persistent kernel (its pencil groups: 16 per warp, N / 16 warps)
 constexpr bool pipeline_supported(int n) { return n % 16 == 0; }

@@ -96,13 +96,13 @@ __global__ void __launch_bounds__(plane_detail::Geo<N, F0>::NT, plane_detail::Ge
     constexpr int W = G::NT / 32;  // warps
     constexpr int GP = 16;         // pencils per warp in pass 1
     static_assert(W * GP == N, "a pass-1 item covers N pencils: N / 16 warps of 16");
-    static_assert((size_t)W * N * GP <= (size_t)N * G::P, "pencil buffers fit the plane tile");
+    static_assert((size_t)W * N * GP <= (size_t)G::E, "pencil buffers fit the plane tile");
     constexpr long long NN = (long long)N * N, N3 = NN * N;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[2 * W];
     __shared__ int s_cur;
     cx<float>* tile = reinterpret_cast<cx<float>*>(smem_raw);
-    cx<float>* tw = tile + N * G::P;
+    cx<float>* tw = tile + G::E;
     for (int j = threadIdx.x; j < N; j += G::NT) tw[j] = reinterpret_cast<const cx<float>*>(a.twx)[j];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long per_step = 3LL * N;

@@ -146,14 +146,16 @@ __device__ __forceinline__ cx<f2> swap_mid(cx<f2> a) {
     return mk(mk_f2(lo(a.re), lo(a.im)), mk_f2(hi(a.re), hi(a.im)));
 }
 
-template <int N, int F0>
+// NAT: the padded natural planes of plane.cuh (pads ride along)
+template <int N, int F0, bool NAT>
 __global__ void __launch_bounds__(32) zline_coulomb(PassArgs a) {
     using PL = CPlan<N, F0>;
     using c2 = cx<f2>;
     static_assert(PL::stages == 2 && N % 2 == 0, "two stages, pencils in pairs");
     constexpr int U = kPairsPerWarp, L = 32 / U;
     constexpr int R0 = PL::radix(0), R1 = PL::radix(1), M0 = N / R0, B1 = N / R1;
-    constexpr long long HU = (long long)N * N / 2;  // pencil pairs of the box
+    constexpr long long HU = (NAT ? plane_elems(N) : N * N) / 2;   // pencil pairs of the box
+    constexpr long long ZU = (NAT ? plane_stride(N) : N * N) / 2;  // ... and from plane to plane
     extern __shared__ __align__(128) unsigned char smem_raw[];
     c2* buf = reinterpret_cast<c2*>(smem_raw);                  // [N][U]
     cx<float>* tw = reinterpret_cast<cx<float>*>(buf + N * U);  // [N]
@@ -164,7 +166,7 @@ __global__ void __launch_bounds__(32) zline_coulomb(PassArgs a) {
     const c2* src = reinterpret_cast<const c2*>(reinterpret_cast<const cx<float>*>(a.src) + t * a.src_tstride) + p;
     if (on)
 #pragma unroll 4
-        for (int z = h; z < N; z += L) cp_async16(buf + z * U + l, src + z * HU);
+        for (int z = h; z < N; z += L) cp_async16(buf + z * U + l, src + z * ZU);
     for (int j = lane; j < N; j += 32) tw[j] = reinterpret_cast<const cx<float>*>(a.twz)[j];
     cp_async_wait();
     __syncwarp();
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(32) zline_coulomb(PassArgs a) {
             f2 k[R1];
             c2 u[R1];
 #pragma unroll
-            for (int q = 0; q < R1; ++q) k[q] = ldg2(kern + (b * R1 + q) * (2 * HU));
+            for (int q = 0; q < R1; ++q) k[q] = ldg2(kern + (b * R1 + q) * (2 * ZU));
 #pragma unroll
             for (int q = 0; q < R1; ++q) u[q] = col[(b * R1 + q) * U];
             Dft<R1, -1, f2>::run(u);
@@ -218,18 +220,17 @@ __global__ void __launch_bounds__(32) zline_coulomb(PassArgs a) {
             }
             Dft<R0, +1, f2>::run(u);
 #pragma unroll
-            for (int s = 0; s < R0; ++s) out[(j + s * M0) * HU] = swap_mid(u[s]);
+            for (int s = 0; s < R0; ++s) out[(j + s * M0) * ZU] = swap_mid(u[s]);
         }
     }
 }
 
 }  // namespace zline_detail
 
-// F0: the first radix of the z axis (0: make_axis_plan's choice)
-template <int N, int F0 = 0>
-cudaError_t zline_launch(const PassArgs& a, int batch, cudaStream_t st) {
+template <int N, int F0, bool NAT>
+cudaError_t zline_launch_nat(const PassArgs& a, int batch, cudaStream_t st) {
     constexpr int U = zline_detail::kPairsPerWarp;
-    auto k = zline_detail::zline_coulomb<N, F0>;
+    auto k = zline_detail::zline_coulomb<N, F0, NAT>;
     static bool carveout = [&] {
         cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaGetLastError();
@@ -237,9 +238,15 @@ cudaError_t zline_launch(const PassArgs& a, int batch, cudaStream_t st) {
     }();
     (void)carveout;
     const size_t smem = (size_t)N * U * sizeof(cx<f2>) + N * sizeof(cx<float>);
-    dim3 grid((unsigned)((N * N / 2 + U - 1) / U), (unsigned)batch);
+    dim3 grid((unsigned)(((NAT ? plane_elems(N) : N * N) / 2 + U - 1) / U), (unsigned)batch);
     k<<<grid, 32, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+// F0: the first radix of the z axis (0: make_axis_plan's choice)
+template <int N, int F0 = 0>
+cudaError_t zline_launch(const PassArgs& a, int batch, cudaStream_t st) {
+    return a.natural ? zline_launch_nat<N, F0, true>(a, batch, st) : zline_launch_nat<N, F0, false>(a, batch, st);
 }
 
 }  // namespace ace
