@@ -169,6 +169,33 @@ __device__ __forceinline__ cx<f2> cmul(cx<f2> a, cx<float> w) {
 }
 #endif
 
+#if defined(__CUDACC__)
+// Four consecutive elements of a plane held in a padded tile, elements 0, 1 at
+// s01, s01 + 1 and 2, 3 at s23, s23 + 1 (a row may end between), read or
+// written by lanes whose vectors follow one another.  The lanes' elements are
+// 4 apart, so lane group i / 4 of a half-warp starts at element (i / 4) % 4 of
+// its own: 16 lanes, 16 bank pairs at every step.
+__device__ __forceinline__ void tile_read4(const cx<float>* tile, int s01, int s23, cx<float> (&v)[4]) {
+    const bool lo = threadIdx.x & 4, hi = threadIdx.x & 8;
+    const int p = hi ? s23 : s01, q = hi ? s01 : s23, o = lo ? 1 : 0;
+    const cx<float> u0 = tile[p + o], u1 = tile[lo ? q : p + 1], u2 = tile[q + o], u3 = tile[lo ? p : q + 1];
+    const cx<float> w0 = lo ? u3 : u0, w1 = lo ? u0 : u1, w2 = lo ? u1 : u2, w3 = lo ? u2 : u3;
+    v[0] = hi ? w2 : w0;
+    v[1] = hi ? w3 : w1;
+    v[2] = hi ? w0 : w2;
+    v[3] = hi ? w1 : w3;
+}
+__device__ __forceinline__ void tile_write4(cx<float>* tile, int s01, int s23, const cx<float> (&v)[4]) {
+    const bool lo = threadIdx.x & 4, hi = threadIdx.x & 8;
+    const int p = hi ? s23 : s01, q = hi ? s01 : s23, o = lo ? 1 : 0;
+    const cx<float> w0 = hi ? v[2] : v[0], w1 = hi ? v[3] : v[1], w2 = hi ? v[0] : v[2], w3 = hi ? v[1] : v[3];
+    tile[p + o] = lo ? w1 : w0;
+    tile[lo ? q : p + 1] = lo ? w2 : w1;
+    tile[q + o] = lo ? w3 : w2;
+    tile[lo ? p : q + 1] = lo ? w0 : w3;
+}
+#endif
+
 // ------------------------------------------------------------------ codelets
 // y_s = sum_q x_q w^{qs}, w = exp(SGN 2 pi i / RAD), in place on v[0..RAD).
 

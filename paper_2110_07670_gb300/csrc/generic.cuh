@@ -130,26 +130,18 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_forward(PassArgs a) {
         const float* fb = reinterpret_cast<const float*>(a.fr) + q.b * N + plane0;
         const float* fc = reinterpret_cast<const float*>(a.fl) + (has2 ? q.c : q.a) * N + plane0;
         const float* fd = reinterpret_cast<const float*>(a.fr) + (has2 ? q.d : q.b) * N + plane0;
-        if (n2 % 4 == 0) {
-            // four columns per load; 16 lanes take 4 rows x 16 columns (lane
-            // (r, c) columns 4c .. 4c + 3 of row r), which the odd pitch spreads
-            // over 16 distinct banks; four steps' loads in flight
-            const int tasks_x = (n2 + 15) / 16, tasks = tasks_x * ((n1 + 3) / 4);
-            const FastDiv dt(tasks_x);
-            const int l = threadIdx.x & 15, hw = threadIdx.x >> 4, nhw = blockDim.x >> 4;
+        if (NN % 4 == 0) {
+            // float4 loads along the plane, whole lines; four steps' in flight
+            const FastDiv dx(n2);
+            const int pad = P - n2;
             constexpr int W = 4;
-            for (int k0 = hw; k0 < tasks; k0 += W * nhw) {
+            for (int k0 = threadIdx.x; k0 < NN / 4; k0 += W * blockDim.x) {
                 V4<float> re[W], im[W];
-                int at[W];
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
-                    const int k = k0 + w * nhw, ty = dt.div(k), y = ty * 4 + (l & 3),
-                              x = (k - ty * tasks_x) * 16 + 4 * (l >> 2);
-                    at[w] = -1;
+                    const int r = 4 * (k0 + w * blockDim.x);
                     im[w] = V4<float>{0.f, 0.f, 0.f, 0.f};
-                    if (k < tasks && y < n1 && x < n2) {
-                        const int r = y * n2 + x;
-                        at[w] = y * P + x;
+                    if (r < NN) {
                         re[w] = ld4(fa + r);
                         if (PRO == PRO_PAIR) re[w] = mul4(re[w], ld4(fb + r));
                         if (has2) {
@@ -160,12 +152,11 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_forward(PassArgs a) {
                 }
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
-                    if (at[w] < 0) continue;
-                    cx<float>* o = tile + at[w];
-                    o[0] = mk(re[w].x, im[w].x);
-                    o[1] = mk(re[w].y, im[w].y);
-                    o[2] = mk(re[w].z, im[w].z);
-                    o[3] = mk(re[w].w, im[w].w);
+                    const int r = 4 * (k0 + w * blockDim.x);
+                    if (r >= NN) continue;
+                    const cx<float> v[4] = {mk(re[w].x, im[w].x), mk(re[w].y, im[w].y), mk(re[w].z, im[w].z),
+                                            mk(re[w].w, im[w].w)};
+                    tile_write4(tile, r + dx.div(r) * pad, r + 2 + dx.div(r + 2) * pad, v);
                 }
             }
         } else {
@@ -265,25 +256,19 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_inverse(PassArgs a) {
     float* wb_p = sym ? reinterpret_cast<float*>(a.accr) + q.b * N + plane0 : nullptr;
     float* wd_p = sym ? reinterpret_cast<float*>(a.accr) + (has2 ? q.d : q.b) * N + plane0 : nullptr;
     float e1 = 0.f, e2 = 0.f;
-    if (n2 % 4 == 0) {
-        // four columns per step, mapped as the forward pass's loads; the loads
-        // of two steps are issued before their updates (ordered operations)
-        const int tasks_x = (n2 + 15) / 16, tasks = tasks_x * ((n1 + 3) / 4);
-        const FastDiv dt(tasks_x);
-        const int l = threadIdx.x & 15, hw = threadIdx.x >> 4, nhw = blockDim.x >> 4;
+    if (NN % 4 == 0) {
+        // four values per step along the plane, every load and reduction in
+        // whole lines; the loads of two steps are issued before their updates
+        // (ordered operations)
+        const FastDiv dx(n2);
+        const int pad = P - n2;
         constexpr int W = 2;
-        for (int k0 = hw; k0 < tasks; k0 += W * nhw) {
+        for (int k0 = threadIdx.x; k0 < NN / 4; k0 += W * blockDim.x) {
             V4<float> la[W], rb[W], lc[W], rd[W];
-            int at[W], rr[W];
 #pragma unroll
             for (int w = 0; w < W; ++w) {
-                const int k = k0 + w * nhw, ty = dt.div(k), y = ty * 4 + (l & 3),
-                          x = (k - ty * tasks_x) * 16 + 4 * (l >> 2);
-                at[w] = -1;
-                if (k < tasks && y < n1 && x < n2) {
-                    const int r = y * n2 + x;
-                    at[w] = y * P + x;
-                    rr[w] = r;
+                const int r = 4 * (k0 + w * blockDim.x);
+                if (r < NN) {
                     la[w] = ld4(la_p + r);
                     rb[w] = ld4(rb_p + r);
                     if (has2) {
@@ -294,10 +279,10 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_inverse(PassArgs a) {
             }
 #pragma unroll
             for (int w = 0; w < W; ++w) {
-                if (at[w] < 0) continue;
-                const int r = rr[w];
-                const cx<float>* src = tile + at[w];
-                const cx<float> v[4] = {src[0], src[1], src[2], src[3]};
+                const int r = 4 * (k0 + w * blockDim.x);
+                if (r >= NN) continue;
+                cx<float> v[4];
+                tile_read4(tile, r + dx.div(r) * pad, r + 2 + dx.div(r + 2) * pad, v);
                 const V4<float> v1 = {v[0].re, v[1].re, v[2].re, v[3].re}, v2 = {v[0].im, v[1].im, v[2].im, v[3].im};
                 V4<float> wa = mul4(v1, rb[w]);
                 e1 += dot4(mul4(la[w], rb[w]), v1);

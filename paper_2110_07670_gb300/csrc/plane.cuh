@@ -384,11 +384,9 @@ __device__ __forceinline__ void inv_accum_plane(const PassArgs& a, const Quad& q
     // vectors, consecutive lanes on consecutive vectors of the plane: every
     // load and every reduction covers whole 128-byte lines.  (Tasks of 4 rows
     // x 16 columns per half-warp, half lines each, took 315 against 224 us per
-    // 64 transforms of 96^3, 119 against 103 at 72^3.)  In the tile a vector's
-    // elements are 4 apart from lane to lane, so lane group i / 4 of a
-    // half-warp starts at element (i / 4) % 4 of its own: 16 lanes, 16 bank
-    // pairs.  (N % 32 == 0: the 16 lanes take 2 rows x 32 columns instead, and
-    // the odd pitch separates the rows: one rotation step less.)
+    // 64 transforms of 96^3, 119 against 103 at 72^3.)  N % 32 == 0: the 16
+    // lanes of a half-warp take 2 rows x 32 columns, and the odd pitch separates
+    // the rows' banks: one rotation step instead of tile_read4's two.
     float e1 = 0.0f, e2 = 0.0f;
     {
         const bool has2 = q.c >= 0, share = has2 && q.c == q.a, sym = a.symmetric != 0;
@@ -406,7 +404,7 @@ __device__ __forceinline__ void inv_accum_plane(const PassArgs& a, const Quad& q
         // issued before the first update
         constexpr int NTASK = N * N / 4, PER = (NTASK + G::NT - 1) / G::NT, U = PER == 1 ? 1 : 2;
         constexpr bool EVEN = PER % U == 0 && NTASK % G::NT == 0;
-        const bool lo = threadIdx.x & 4, hi = threadIdx.x & 8;
+        const bool odd4 = threadIdx.x & 4;
         for (int k0 = 0; k0 < PER; k0 += U) {
             float4 la[U], rb[U], lc[U], rd[U];
             int rof[U], s01[U], s23[U];  // offsets in the plane; of elements 0, 1 and 2, 3 in the tile
@@ -441,21 +439,14 @@ __device__ __forceinline__ void inv_accum_plane(const PassArgs& a, const Quad& q
                 const int r = rof[u];
                 cx<float> v[4];
                 if constexpr (TWO_ROWS) {
-                    const int p = lo ? s23[u] : s01[u], q2 = lo ? s01[u] : s23[u];
+                    const int p = odd4 ? s23[u] : s01[u], q2 = odd4 ? s01[u] : s23[u];
                     const cx<float> w0 = tile[p], w1 = tile[p + 1], w2 = tile[q2], w3 = tile[q2 + 1];
-                    v[0] = lo ? w2 : w0;
-                    v[1] = lo ? w3 : w1;
-                    v[2] = lo ? w0 : w2;
-                    v[3] = lo ? w1 : w3;
+                    v[0] = odd4 ? w2 : w0;
+                    v[1] = odd4 ? w3 : w1;
+                    v[2] = odd4 ? w0 : w2;
+                    v[3] = odd4 ? w1 : w3;
                 } else {
-                    const int p = hi ? s23[u] : s01[u], q2 = hi ? s01[u] : s23[u], o = lo ? 1 : 0;
-                    const cx<float> u0 = tile[p + o], u1 = tile[lo ? q2 : p + 1], u2 = tile[q2 + o],
-                                    u3 = tile[lo ? p : q2 + 1];
-                    const cx<float> w0 = lo ? u3 : u0, w1 = lo ? u0 : u1, w2 = lo ? u1 : u2, w3 = lo ? u2 : u3;
-                    v[0] = hi ? w2 : w0;
-                    v[1] = hi ? w3 : w1;
-                    v[2] = hi ? w0 : w2;
-                    v[3] = hi ? w1 : w3;
+                    tile_read4(tile, s01[u], s23[u], v);
                 }
                 const float4 v1 = make_float4(v[0].re, v[1].re, v[2].re, v[3].re);
                 const float4 v2 = make_float4(v[0].im, v[1].im, v[2].im, v[3].im);

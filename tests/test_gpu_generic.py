@@ -21,7 +21,7 @@ def rel(a, b):
 
 
 @pytest.mark.parametrize("grid", [(15, 9, 25), (27, 45, 15), (20, 16, 18), (9, 8, 250), (250, 10, 12), (5, 162, 6),
-                                  (12, 75, 54), (6, 5, 4 * 27)])
+                                  (12, 75, 54), (6, 5, 4 * 27), (10, 12, 15)])
 @pytest.mark.parametrize("cut", [False, True])
 def test_generic_boxes_match_oracle(grid, cut):
     import torch
