@@ -133,6 +133,8 @@ struct ace_plan {
         int* ipiv = nullptr;      // pivots [n], status
         size_t c_dpsi = 0, c_dens = 0, c_isel = 0, c_A = 0, c_nu = 0, c_part = 0, c_mats = 0, c_ipiv = 0;
     } scdm;
+    double fft_gain = 1;       // mean gain of the orbital and W transforms (axis_gain; single precision)
+    double pair_gain = 1;      // ... and of the pair passes' transforms, under their radix plan
     int variant = 1;           // pair passes: 1 tile, 2 transposed planes, 3 persistent pipeline, 4 hybrid
     bool hybrid = false;       // variant 4: plane kernels with padded natural planes
     bool half = false;         // variant 5: P1 / P3 on clusters of two half-plane blocks (halfplane.cuh)
@@ -358,6 +360,69 @@ int setup_shapes(ace_plan* P) {
     return ACE_OK;
 }
 
+// A real that rounds constants to single precision and computes in double.
+struct RoundedConst {
+    double v;
+    RoundedConst() = default;
+    RoundedConst(double c) : v((float)c) {}
+    static RoundedConst of(double x) {
+        RoundedConst r;
+        r.v = x;
+        return r;
+    }
+};
+inline RoundedConst operator+(RoundedConst a, RoundedConst b) { return RoundedConst::of(a.v + b.v); }
+inline RoundedConst operator-(RoundedConst a, RoundedConst b) { return RoundedConst::of(a.v - b.v); }
+inline RoundedConst operator*(RoundedConst a, RoundedConst b) { return RoundedConst::of(a.v * b.v); }
+inline RoundedConst operator-(RoundedConst a) { return RoundedConst::of(-a.v); }
+
+template <int RAD>
+double codelet_gain() {
+    double sum = 0;
+    for (int q = 0; q < RAD; ++q) {
+        cx<RoundedConst> v[RAD];
+        for (int k = 0; k < RAD; ++k) v[k] = mk(RoundedConst::of(k == q), RoundedConst::of(0));
+        Dft<RAD, -1, RoundedConst>::run(v);
+        for (int s = 0; s < RAD; ++s) {
+            const double t = -2 * M_PI * (q * s % RAD) / RAD;
+            sum += v[s].re.v * std::cos(t) + v[s].im.v * std::sin(t);
+        }
+    }
+    return sum / (RAD * RAD);
+}
+
+// Mean gain of one axis in single precision: the part of its transform's
+// error that a rounded constant (codelet or twiddle) makes common to every
+// value, Re tr(F^H F~) / n to first order stage by stage.
+double axis_gain(const AxisPlan& p) {
+    double g = 1;
+    int len = p.n;  // block length of the stage
+    for (int st = 0; st < p.nstages; ++st) {
+        const int rad = p.radix[st], m = len / rad;
+        switch (rad) {
+            case 3: g *= codelet_gain<3>(); break;
+            case 5: g *= codelet_gain<5>(); break;
+            case 6: g *= codelet_gain<6>(); break;
+            case 8: g *= codelet_gain<8>(); break;
+            case 9: g *= codelet_gain<9>(); break;
+            case 10: g *= codelet_gain<10>(); break;
+            case 12: g *= codelet_gain<12>(); break;
+            case 15: g *= codelet_gain<15>(); break;
+            case 16: g *= codelet_gain<16>(); break;
+            default: break;  // 2 and 4 are exact
+        }
+        double tw = 0;
+        for (int s = 0; s < rad; ++s)
+            for (int j = 0; j < m; ++j) {
+                const double t = 2 * M_PI * s * j / len, c = std::cos(t), w = std::sin(t);
+                tw += c * (float)c + w * (float)w;
+            }
+        g *= tw / len;
+        len = m;
+    }
+    return g;
+}
+
 template <typename R>
 PassArgs base_args(const ace_plan* P) {
     PassArgs a;
@@ -374,7 +439,7 @@ PassArgs base_args(const ace_plan* P) {
     a.src_tstride = a.dst_tstride = P->N;
     a.src = a.dst = P->d_spec;
     for (int i = 0; i < 9; ++i) a.b[i] = P->b[i];
-    a.kscale = 1.0 / (double)P->N;
+    a.kscale = 1.0 / (double)P->N / (P->pair_gain * P->pair_gain);
     a.err = P->d_err;
     a.lookahead = P->lookahead;
     a.kern = P->tplane ? P->d_kern_t : P->d_kern;
@@ -392,12 +457,13 @@ PassArgs base_args(const ace_plan* P) {
     } while (0)
 
 // The real-space functions of run_to_real are psi(r) times this number: the
-// scale Omega^-1/2 rounded to the plan's precision, over itself.  A coherent
-// error of up to 6e-8 per function in single precision; the factors applied to
-// products of functions afterwards (in double) divide it out again.
+// scale Omega^-1/2 rounded to the plan's precision, over itself, and the mean
+// gain of the transform's rounded constants (axis_gain).  Coherent errors of
+// up to 6e-8 per function in single precision; the factors applied to
+// products of functions afterwards (in double) divide them out again.
 template <typename R>
 double phi_gain(const ace_plan* P) {
-    return (double)(R)(1.0 / std::sqrt(P->omega)) * std::sqrt(P->omega);
+    return (double)(R)(1.0 / std::sqrt(P->omega)) * std::sqrt(P->omega) * P->fft_gain;
 }
 
 // psi (half sphere) -> real-space functions out[a] (quads (a, a, c, c)).
@@ -452,7 +518,7 @@ int run_to_recip(ace_plan* P, const R* acc, const Quad* dq, int ntrans, double s
             ACE_CKL(sphere_launch(a, P->sp, false, nb, st));
         else
             ACE_CKL(launch_pass<R>(a, P->s_z, PRO_LOAD, EPI_STORE, MID_NONE, -1, nb, st));
-        ACE_CKL(launch_gather<R>(spec, dq, t0, nb, P->npw, P->d_ip, P->d_in, P->N, s, out, st));
+        ACE_CKL(launch_gather<R>(spec, dq, t0, nb, P->npw, P->d_ip, P->d_in, P->N, s / P->fft_gain, out, st));
     }
     return ACE_OK;
 }
@@ -1507,16 +1573,20 @@ double auxiliary_function_k0(const double cell[9], const double b[9], double ome
 template <typename R>
 int pair_tables(ace_plan* P, int r0) {
     std::vector<int> frq[3];
+    double gain = 1;
     for (int d = 0; d < 3; ++d) {
         AxisPlan ax = P->ax[d];
         if (r0 != 0 && !make_axis_plan_first(P->n[d], r0, ax))
             return fail(ACE_ERR_INVALID_ARG, "pair radix plan: the radix does not split the grid into two codelets");
+        if (sizeof(R) == 4) gain *= axis_gain(ax);
         frq[d].resize(P->n[d]);
         for (int k = 0; k < P->n[d]; ++k) frq[d][digit_reversed_position(ax, k)] = k;
         if (!P->d_freq[d]) ACE_TRY(dalloc((void**)&P->d_freq[d], P->n[d] * sizeof(int)));
         ACE_CK(cudaMemcpy(P->d_freq[d], frq[d].data(), P->n[d] * sizeof(int), cudaMemcpyHostToDevice));
     }
     P->pair_r0 = r0;
+    P->pair_gain = gain;
+    if (r0 == 0) P->fft_gain = gain;
     const bool swz = P->s_xy.cube && cube_swizzle(P->n[2]);
     const bool tab = P->zline || P->gen;
     const bool inline_tab = !tab && (P->coul_rc > 0 || P->coul_g0 || sizeof(R) == 8);
@@ -1539,11 +1609,12 @@ int pair_tables(ace_plan* P, int r0) {
     };
     // 4 pi / |G|^2 with G = 0 dropped, or the transform of 1/r cut off at
     // R_c: 4 pi (1 - cos(|G| R_c)) / |G|^2, and 2 pi R_c^2 at G = 0
-    const double rc = P->coul_rc;
+    // (over N and the gains of a forward and an inverse transform)
+    const double rc = P->coul_rc, nn = (double)P->N * gain * gain;
     auto k = [&](double q2) {
         if (rc > 0)
-            return (q2 > 0 ? 4 * M_PI * (1 - std::cos(std::sqrt(q2) * rc)) / q2 : 2 * M_PI * rc * rc) / (double)P->N;
-        return q2 > 0 ? 4 * M_PI / (q2 * (double)P->N) : P->coul_k0 / (double)P->N;
+            return (q2 > 0 ? 4 * M_PI * (1 - std::cos(std::sqrt(q2) * rc)) / q2 : 2 * M_PI * rc * rc) / nn;
+        return q2 > 0 ? 4 * M_PI / (q2 * nn) : P->coul_k0 / nn;
     };
     for (int z = 0; z < n0; ++z)
         for (int y = 0; y < n1; ++y)

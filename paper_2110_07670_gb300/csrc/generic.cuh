@@ -22,7 +22,7 @@
 // kernels' instructions per element).  Against the runtime-size tile passes these
 // replace, per 32 transforms of 72^3: forward planes 62 vs 127 us, pencils 48 vs
 // 347, inverse planes 93 vs 150; 64 orbitals there 6.4 vs 19.8 ms per build, 27
-// orbitals on 40 x 48 x 45 0.58 vs 1.28 ms.
+// orbitals on 40 x 48 x 45 0.50 vs 1.31 ms.
 #pragma once
 
 #include "internal.h"
