@@ -256,13 +256,11 @@ def pass_bytes(n, N, esz=4, batch=64):
     return tot, launches
 
 
-# DRAM bytes per launch (64 transforms) of the pair passes on this workload,
-# from ncu captures (dram__bytes_read.sum + dram__bytes_write.sum; see
-# profiles/dram_pair_passes_water32_96cubed.md): the tile-pass forward kernel,
-# the plane-kernel forward pass of the hybrid variant, and the Coulomb and
-# accumulation kernels both variants share.
-MEASURED_TRAFFIC_PER_LAUNCH = {"pair_fwd": None, "pair_fwd_hybrid": 0.5473e9, "pair_coulomb": 0.8473e9,
-                               "pair_inv": 0.8595e9}
+# DRAM bytes per launch (64 transforms) of the hybrid variant's passes on this
+# workload, from ncu captures (dram__bytes_read.sum + dram__bytes_write.sum; see
+# profiles/dram_pair_passes_water32_96cubed.md).
+MEASURED_TRAFFIC_PER_LAUNCH = {"pair_fwd": None, "pair_fwd_hybrid": 0.5512e9, "pair_coulomb": 0.8576e9,
+                               "pair_inv": 0.8646e9}
 
 
 def cpu_baseline(cfg, rows=5):
@@ -423,7 +421,7 @@ def run_ours(args):
     kcfg = plan.config()
     variant, streams = kcfg["pair_variant"], kcfg["pair_streams"]
     vname = {1: "tile passes", 2: "transposed-plane passes", 3: "persistent pipeline kernel",
-             4: "plane-kernel forward pass, tile passes after it",
+             4: "plane kernels on natural planes",
              5: "plane passes on clusters of two half-plane blocks"}[variant]
     group = 32 if (variant != 3 and streams == 2) else 64  # transforms per launch (algorithmic count)
     pbg, _ = pass_bytes(n, N, batch=group)

@@ -78,7 +78,7 @@ typedef struct {
                           1 = every pass in order on the call's stream */
     int pair_variant;  /* kernels of the pair passes (Eq. 2-4): 1 tile passes, 2 transposed-
                           plane passes, 3 one persistent kernel for all three passes, 4 the
-                          plane-kernel forward pass with the tile passes after it, 5 the
+                          plane kernels with their padded planes as the spectrum, 5 the
                           plane passes on clusters of two blocks holding half a plane each
                           (2: single precision, n^3 boxes with n in {32, 80, 96, 120, 160};
                           3: single precision, n in {32, 80, 96, 160};

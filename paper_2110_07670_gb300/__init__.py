@@ -219,7 +219,7 @@ def ace_plan_create(grid, cell, ecut, n_occ_max, precision="mixed", pair_batch=0
     """kernels: 0 fastest available, 1 CUDA-core Gram products, 2 also generic FFT passes;
     pair_streams: 0 automatic, 1 every pair pass in order on the call's stream;
     pair_variant: 0 automatic (timed at creation), 1 tile passes, 2 transposed planes,
-    3 persistent pipeline, 4 hybrid (plane-kernel forward pass, tile passes after it);
+    3 persistent pipeline, 4 hybrid (plane kernels, the padded planes as the spectrum);
     coulomb_rc: 0 bare Coulomb with G = 0 dropped, > 0 the interaction cut off at that radius;
     coulomb_g0: keep the bare kernel's G = 0 term as the auxiliary-function value."""
     return Plan(grid, cell, ecut, n_occ_max, precision, pair_batch, kernels, pair_streams, pair_variant, coulomb_rc,
