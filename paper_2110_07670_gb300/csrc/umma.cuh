@@ -94,11 +94,14 @@ __device__ __forceinline__ uint32_t tf32_round(float x) {
 // x = hi + lo + O(2^-22 |x|): hi = tf32(x), lo = tf32(x - hi), by integer
 // rounding (half away from zero).  The tensor cores read the upper 19 bits of an
 // operand, so lo is left with its rounding carry added and its low bits in
-// place.  (Four ALU operations; with two conversions the Gram's stages took 10%
-// longer.)
+// place.  The carry turns an all-ones NaN (the one that device arithmetic makes)
+// into a zero, so hi takes 0 * (x - hi) on top: NaN where x is NaN or infinite,
+// nothing otherwise.  (Five operations; with two conversions the Gram's stages
+// took 10% longer.)
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
-    lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
+    const float h = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u), r = x - h;
+    hi = __float_as_uint(fmaf(r, 0.0f, h));
+    lo = __float_as_uint(r) + 0x1000u;
 }
 
 // Byte offset of element (row, k) (k < 32) of a K-major tile of 32-value rows
