@@ -142,17 +142,25 @@ __device__ __forceinline__ void ws_mma(WsSmem& sm, int buf, uint32_t tmem, int s
     }
 }
 
-// The accumulators truncate: a sum of one sign loses on average half an ulp of
-// its running value per K step (and alignment bits inside a step), over the 8
-// steps of a turn 2.5e-7 of the turn's sum (from the errors of M, E and K psi
-// against FP64 on 72^3 to 160^3 builds).  The drain's add is a fused
-// multiply-add with 1 + 2^-22 = 1 + 2.4e-7 instead, at the same cost.
-constexpr float kTruncGain = 1.0f + 0x1p-22f;
+// The accumulators truncate: a K step takes about 2^-25 of the sum away.
+// Measured (128 x 128 products against FP64, means over the entries, e-8 after
+// 1, 2, 4 and 8 steps): uniform in [0.5, 1] 2.3, 5.0, 9.1, 22; |normal| 3.9, 6.5,
+// 13, 29; of either sign, as a part of the result, 3.7, 5.3, 8.8, 15.  The drain
+// gives back one ulp of one, 2^-23, for each stage of the turn that is full of data
+// (4 steps), in a fused multiply-add that costs what the add did; a stage that
+// is not full gets nothing, steps of zeros lose nothing.  What is left is below
+// 1.4e-7 of a turn's sum (7 steps), and 6e-8 of a full one's.  (Where a row is
+// zero but for a few values of a turn, up to 2.1e-7 is gained.)
+constexpr float kFullGain = 1.0f + DS * 0x1p-23f;
+__device__ __forceinline__ float last_gain(long long K) {  // of the last turn of K values
+    return 1.0f + (float)(((int)((K - 1) % (DS * TK)) + 1) / TK) * 0x1p-23f;
+}
 
 // A drain warp's share of accumulator set `set`: its TMEM lane quarter (warp
 // % 4) and its 64 columns ((warp - 8) / 4), added (or, first, stored) into
-// sum[64] as hi.hi + small; then the set is released.
-__device__ __forceinline__ void ws_drain(WsSmem& sm, uint32_t tmem, int set, bool first, float (&sum)[64]) {
+// sum[64] as gain hi.hi + small; then the set is released.
+__device__ __forceinline__ void ws_drain(WsSmem& sm, uint32_t tmem, int set, bool first, float gain,
+                                         float (&sum)[64]) {
     const int warp = threadIdx.x >> 5;
     const uint32_t taddr = tmem + (uint32_t)set * 256 + ((uint32_t)((warp & 3) * 32) << 16) +
                            (uint32_t)(((warp - WARP_DRAIN0) >> 2) * 64);
@@ -164,7 +172,7 @@ __device__ __forceinline__ void ws_drain(WsSmem& sm, uint32_t tmem, int set, boo
         umma::tmem_wait_ld();
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-            const float x = fmaf(__uint_as_float(v[c]), kTruncGain, __uint_as_float(w[c]));
+            const float x = fmaf(__uint_as_float(v[c]), gain, __uint_as_float(w[c]));
             sum[16 * h + c] = first ? x : sum[16 * h + c] + x;
         }
     }
@@ -264,6 +272,7 @@ __global__ void __launch_bounds__(NTHR, 1)
             return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
         };
         const bool issuer = warp == WARP_DRAIN0;
+        const float lgain = last_gain(k1 - k0);
         float sum[64];
         bool ok = !issuer || nturn == 0 || issue_turn(0);
         for (int q = 0; q < nturn && ok; ++q) {
@@ -271,7 +280,7 @@ __global__ void __launch_bounds__(NTHR, 1)
             if (ok) ok = ws_wait(sm, &sm.tfull[q & 1], q / 2, err);
             if (ok) {
                 umma::fence_after_sync();
-                ws_drain(sm, tmem, q & 1, q == 0, sum);
+                ws_drain(sm, tmem, q & 1, q == 0, q + 1 < nturn ? kFullGain : lgain, sum);
             }
         }
         // the MMAs in flight finish before the block releases TMEM
@@ -439,6 +448,7 @@ __global__ void __launch_bounds__(NTHR, 1)
             return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
         };
         const bool issuer = warp == WARP_DRAIN0;
+        const float lgain = last_gain(n);
         float sum[64];
         const int jl = (warp & 3) * 32 + (threadIdx.x & 31);
         const int tc = ((warp - WARP_DRAIN0) >> 2) * 64;
@@ -448,7 +458,7 @@ __global__ void __launch_bounds__(NTHR, 1)
             if (!ok || !ws_wait(sm, &sm.tfull[q & 1], q / 2, err)) break;
             umma::fence_after_sync();
             const int sub = (int)(q % nsub);
-            ws_drain(sm, tmem, (int)(q & 1), sub == 0, sum);
+            ws_drain(sm, tmem, (int)(q & 1), sub == 0, sub < nsub - 1 ? kFullGain : lgain, sum);
             if (sub == nsub - 1) {  // the tile is complete
                 const int tile = blockIdx.x + (int)(q / nsub) * G;
                 const long long j = (long long)(tile / ntb) * 128 + jl;
