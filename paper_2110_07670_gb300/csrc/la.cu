@@ -147,10 +147,11 @@ __global__ void gram_finish_kernel(const PT* __restrict__ P, int nchunk, const R
 // The same from single-precision partials with many K slices: a block owns
 // 32 consecutive columns (one per lane) of one row and its eight warps sum
 // interleaved eighths of the slices (four loads in flight each), combined in a
-// fixed order.  A warp's sums are float-float (TwoSum, about 2^-46 of the sum of
-// magnitudes): converting and adding every partial in double kept the FP64 pipe
-// 71% busy (17 us for 144 slices of 128 x 128).  What the finished element G_ij
-// becomes:
+// fixed order.  The sums are kept in three floats (sum_add3, 2^-64 of the sum of
+// magnitudes: below a sum in double) on the FP32 pipes: converting and adding
+// every partial in double kept the FP64 pipe 71% busy (17 us for 144 slices of
+// 128 x 128).  Where they leave the range of a float, in double after all.  What
+// the finished element G_ij becomes:
 //   FIN_MATRIX  G[i][j]
 //   FIN_IMAGE   the apply product's operand image of C = G: TF32 hi / lo in the
 //               swizzled tiles of launch_apply_product, zero outside m x n (the
@@ -158,10 +159,21 @@ __global__ void gram_finish_kernel(const PT* __restrict__ P, int nchunk, const R
 //   FIN_SUMSQ   sum over the block's columns of G_ij^2 (the fast MTS energy)
 enum GramFinish { FIN_MATRIX = 0, FIN_IMAGE = 1, FIN_SUMSQ = 2 };
 
-__device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
-    const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
-    hi = t;
+// (s, e, ee) += x: TwoSum's error goes to e by a TwoSum of its own, whose error is
+// added up in ee (A. Klein, A generalized Kahan-Babuska-summation algorithm,
+// Computing 76 (2006)).
+__device__ __forceinline__ float two_sum(float& s, float x) {
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+    s = t;
+    return e;
+}
+__device__ __forceinline__ void sum_add3(float& s, float& e, float& ee, float x) {
+    ee = __fadd_rn(ee, two_sum(e, two_sum(s, x)));
+}
+__device__ __forceinline__ void sum_merge3(float& s, float& e, float& ee, float s2, float e2, float ee2) {
+    sum_add3(s, e, ee, s2);
+    ee = __fadd_rn(ee, __fadd_rn(two_sum(e, e2), ee2));
 }
 
 template <int FIN>
@@ -170,13 +182,13 @@ __global__ void __launch_bounds__(256) gram_finish_f32_kernel(const float* __res
                                                               const float* __restrict__ B, int m, int n, long long K,
                                                               double* __restrict__ G, int ldg,
                                                               float* __restrict__ img) {
-    __shared__ double part[8][32];
+    __shared__ float part[3][8][32];
     const long long tot = (long long)m * n;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x, j = blockIdx.y * 32 + lane;
     const bool in = i < m && j < n;
     const long long e = (long long)i * n + j;
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    float s0[4] = {}, s1[4] = {}, s2[4] = {};
     if (in) {
         int c = w;
         for (; c + 24 < nchunk; c += 32) {
@@ -184,21 +196,26 @@ __global__ void __launch_bounds__(256) gram_finish_f32_kernel(const float* __res
 #pragma unroll
             for (int u = 0; u < 4; ++u) v[u] = P[(long long)(c + 8 * u) * tot + e];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) ff_add(hi[u], lo[u], v[u]);
+            for (int u = 0; u < 4; ++u) sum_add3(s0[u], s1[u], s2[u], v[u]);
         }
-        for (; c < nchunk; c += 8) ff_add(hi[0], lo[0], P[(long long)c * tot + e]);
+        for (; c < nchunk; c += 8) sum_add3(s0[0], s1[0], s2[0], P[(long long)c * tot + e]);
 #pragma unroll
-        for (int u = 1; u < 4; ++u) {
-            ff_add(hi[0], lo[0], hi[u]);
-            lo[0] = __fadd_rn(lo[0], lo[u]);
-        }
+        for (int u = 1; u < 4; ++u) sum_merge3(s0[0], s1[0], s2[0], s0[u], s1[u], s2[u]);
     }
-    part[w][lane] = (double)hi[0] + (double)lo[0];
+    part[0][w][lane] = s0[0];
+    part[1][w][lane] = s1[0];
+    part[2][w][lane] = s2[0];
     __syncthreads();
     if (w != 0) return;
     double g = 0.0;
     if (in) {
-        for (int k = 0; k < 8; ++k) g += part[k][lane];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) sum_merge3(s0[0], s1[0], s2[0], part[0][k][lane], part[1][k][lane], part[2][k][lane]);
+        g = (double)s0[0] + ((double)s1[0] + (double)s2[0]);
+        if (!isfinite(s0[0])) {
+            g = 0.0;
+            for (int c = 0; c < nchunk; ++c) g += (double)P[(long long)c * tot + e];
+        }
         const double g0 = double(A[(long long)i * K]) * double(B[(long long)j * K]) +
                           double(A[(long long)i * K + 1]) * double(B[(long long)j * K + 1]);
         g = 2.0 * g - g0;

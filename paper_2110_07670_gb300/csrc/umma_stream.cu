@@ -5,7 +5,7 @@
 //   Gram     G[i][j] = sum_k A[i][k] B[j][k] over K = 2 n_pw_half reals
 //            (C = psi^T xi of the apply, M = Phi^T W of the build), as FP32
 //            partials over K slices (about one block per SM) that
-//            launch_gram_finish_f32 sums in FP64;
+//            launch_gram_finish_f32 sums as precisely as FP64 would;
 //   product  out[t][j] = -sum_k C[t][k] xi[k][j]  (K psi = -xi C^T), with C
 //            the apply's Gram, split to TF32 hi / lo beforehand.
 //
