@@ -1,6 +1,7 @@
 // la.cu -- sphere scatter/gather, Gamma-point Gram products, the dense
 // products of the ACE construction and apply, the FP64 Cholesky, and the
 // exchange-energy reduction (arXiv:2110.07670 Section 2.2 and Eq. 4-5).
+#include "float_sums.cuh"
 #include "internal.h"
 #include "tma.cuh"
 #include "umma.cuh"
@@ -158,23 +159,6 @@ __global__ void gram_finish_kernel(const PT* __restrict__ P, int nchunk, const R
 //               grid covers the padded tiles)
 //   FIN_SUMSQ   sum over the block's columns of G_ij^2 (the fast MTS energy)
 enum GramFinish { FIN_MATRIX = 0, FIN_IMAGE = 1, FIN_SUMSQ = 2 };
-
-// (s, e, ee) += x: TwoSum's error goes to e by a TwoSum of its own, whose error is
-// added up in ee (A. Klein, A generalized Kahan-Babuska-summation algorithm,
-// Computing 76 (2006)).
-__device__ __forceinline__ float two_sum(float& s, float x) {
-    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
-    s = t;
-    return e;
-}
-__device__ __forceinline__ void sum_add3(float& s, float& e, float& ee, float x) {
-    ee = __fadd_rn(ee, two_sum(e, two_sum(s, x)));
-}
-__device__ __forceinline__ void sum_merge3(float& s, float& e, float& ee, float s2, float e2, float ee2) {
-    sum_add3(s, e, ee, s2);
-    ee = __fadd_rn(ee, __fadd_rn(two_sum(e, e2), ee2));
-}
 
 template <int FIN>
 __global__ void __launch_bounds__(256) gram_finish_f32_kernel(const float* __restrict__ P, int nchunk,

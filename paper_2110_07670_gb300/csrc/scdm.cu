@@ -11,14 +11,14 @@
 //   Phi = (V V^T)^{-1/2} V Psi, V[k][i] = psi_i(r_{C_k}): the polar factor of V
 //     by scaled Newton-Schulz steps X <- X (3 I - X^T X) / 2 from V / |V|_F
 // Sums and decisions in double; the orbitals' real-space values come in the
-// plan's precision, and for single precision the QR's column pass (and, up to 256
-// orbitals, its projections) form their products in float-float arithmetic
-// (about 2^-46 relative) on the FP32 pipes.
+// plan's precision, and for single precision the QR's column pass forms its
+// products in float-float arithmetic (about 2^-48 relative) on the FP32 pipes.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <type_traits>
 
+#include "float_sums.cuh"
 #include "internal.h"
 
 namespace ace {
@@ -370,79 +370,58 @@ __device__ __forceinline__ void ff_dot_acc(float qh, float ql, float a, float& s
     sh = s;
 }
 
-// Single precision and n <= kPivotN: (1) and (2) and the normalisation in one
-// block, in float-float arithmetic on the FP32 pipes like the column pass (one
-// SM's FP64 rate, two multiply-adds per cycle, would take 12 us for 128 orbitals;
-// spread over blocks it took three launches, 14 us, and every block of the column
-// pass then repeated the norm, root and split).  Measured for 128 orbitals: 9.6
-// us per step, the column pass 6.8 instead of 13.6, the whole call 5.5 instead of
-// 7.6 ms.  Bound by the latency of its serial parts.  Above kPivotN orbitals one
-// SM falls behind the spread form.  q_k goes out as two floats, Q [n][2][n].
-constexpr int kPivotN = 256, kPivotThreads = 512;
+// Single precision and n <= kPivotN: (1), (2) and the normalisation in one block.
+// The coefficients of the first projection are formed here, in double, and not
+// taken from the column pass's rows of R, whose float-float products would leave
+// q_k orthogonal to 2^-47 only, and so is the length that decides on the second
+// one.  Bound by one SM's FP64 rate (two multiply-adds per cycle) and the latency
+// of its serial parts.  A whole step (with the column pass, 22,000 columns): 14.3,
+// 18.5, 24 us for 8, 64, 128 orbitals, where the form spread over blocks (three
+// launches, every block of the column pass repeating the norm, root and split)
+// takes 20, 24.5, 28; at 192 it is 35 against 31, so the line lies between.  q_k
+// goes out in double and, for the column pass, as the float pairs qs [2][n].
+constexpr int kPivotN = 160, kPivotThreads = 512;
 
-// (sh, sl) += (h, l)
-__device__ __forceinline__ void ff_pair_add(float& sh, float& sl, float h, float l) {
-    const float s = __fadd_rn(sh, h), bb = __fsub_rn(s, sh);
-    sl = __fadd_rn(__fadd_rn(sl, l), __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(h, bb)));
-    sh = s;
+// (s, e, ee) += h + l
+__device__ __forceinline__ void sum_pair3(float& s, float& e, float& ee, float h, float l) {
+    const float e1 = two_sum(s, h), e2 = two_sum(e, l);
+    ee = __fadd_rn(ee, __fadd_rn(e2, two_sum(e, e1)));
 }
 
-// sum += c q for c = ch + cl, q = qh + ql (float pairs), kept as the pair (sh, sl)
-__device__ __forceinline__ void ff_mul_acc(float ch, float cl, float qh, float ql, float& sh, float& sl) {
-    const float p = __fmul_rn(ch, qh);
-    float e = fmaf(ch, qh, -p);  // ch qh - p, exactly
-    e = fmaf(ch, ql, e);
-    e = fmaf(cl, qh, e);
-    const float s = __fadd_rn(sh, p), bb = __fsub_rn(s, sh);
-    const float t = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    sl = __fadd_rn(sl, __fadd_rn(t, e));
-    sh = s;
-}
-
-// r[i] -= sum_{l < k} (ch + cl)[l] q_l[i] by the whole block (n <= blockDim); the
-// sums stay float pairs, one double subtraction per row ends them
-__device__ __forceinline__ void subtract_projections(double* r, const float* ch, const float* cl,
-                                                     const float* __restrict__ Q, int n, int k, float2* part) {
-    const int groups = blockDim.x / n, g = threadIdx.x / n, i = threadIdx.x - g * n;
+// r[i] -= sum_{l < k} c[l] q_l[i] by the whole block (k < n <= blockDim)
+__device__ __forceinline__ void subtract_projections(double* r, const double* c, const double* __restrict__ Q, int n,
+                                                     int k, double* part) {
+    const int groups = min((int)blockDim.x / n, k), g = threadIdx.x / n, i = threadIdx.x - g * n;
     if (g < groups) {
-        float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
-        const float* q = Q + i;
-        // eight rows' loads in flight (past k: zeros)
+        double s[2] = {0, 0};
+        // eight rows' loads in flight
         for (int l = g; l < k; l += 8 * groups) {
-            float qh[8], ql[8];
+            double q[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const bool in = l + u * groups < k;
-                qh[u] = in ? q[(l + u * groups) * 2 * n] : 0.f;
-                ql[u] = in ? q[(l + u * groups) * 2 * n + n] : 0.f;
-            }
+            for (int u = 0; u < 8; ++u) q[u] = l + u * groups < k ? Q[(l + u * groups) * n + i] : 0.0;
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (l + u * groups < k)
-                    ff_mul_acc(ch[l + u * groups], cl[l + u * groups], qh[u], ql[u], sh[u & 3], sl[u & 3]);
+                if (l + u * groups < k) s[u & 1] += c[l + u * groups] * q[u];
         }
-#pragma unroll
-        for (int u = 1; u < 4; ++u) ff_pair_add(sh[0], sl[0], sh[u], sl[u]);
-        part[g * n + i] = make_float2(sh[0], sl[0]);
+        part[g * n + i] = s[0] + s[1];
     }
     __syncthreads();
     if ((int)threadIdx.x < n) {
-        float h = 0.f, l = 0.f;
-        for (int gg = 0; gg < groups; ++gg) ff_pair_add(h, l, part[gg * n + threadIdx.x].x, part[gg * n + threadIdx.x].y);
-        r[threadIdx.x] -= (double)h + (double)l;
+        double t = 0;
+        for (int gg = 0; gg < groups; ++gg) t += part[gg * n + threadIdx.x];
+        r[threadIdx.x] -= t;
     }
     __syncthreads();
 }
 
 __global__ void __launch_bounds__(kPivotThreads) qr_pivot_kernel(const ArgMax* __restrict__ parts, int nparts,
                                                                  const float* __restrict__ A, int n, long long m,
-                                                                 const double* __restrict__ Rrows, int k,
-                                                                 float* __restrict__ Q, int* __restrict__ piv,
-                                                                 double* __restrict__ nu, double* __restrict__ nu0,
-                                                                 double* __restrict__ rdiag, int* __restrict__ status) {
-    __shared__ double r[kPivotN], s_inv;
-    __shared__ float2 part[kPivotThreads];
-    __shared__ float ch[kPivotN], cl[kPivotN], rh[kPivotN], rl[kPivotN];
+                                                                 int k, double* Q, float* __restrict__ qs,
+                                                                 int* __restrict__ piv, double* __restrict__ nu,
+                                                                 double* __restrict__ nu0, double* __restrict__ rdiag,
+                                                                 int* __restrict__ status) {
+    __shared__ double r[kPivotN], c[kPivotN], part[kPivotThreads], s_inv;
+    __shared__ double norm2[2];  // |a_p|^2, |r|^2
     __shared__ ArgMax wbest[kPivotThreads / 32];
     __shared__ long long s_p;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -480,104 +459,86 @@ __global__ void __launch_bounds__(kPivotThreads) qr_pivot_kernel(const ArgMax* _
     __syncthreads();
     const long long p = s_p;
     if (p < 0) {  // rank deficient: a zero row
-        for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) Q[(long long)k * 2 * n + i] = 0.f;
+        for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) {
+            if (i < n) Q[(long long)k * n + i] = 0.0;
+            qs[i] = 0.f;
+        }
         if (threadIdx.x == 0) rdiag[k] = 0.0;
         return;
     }
-    for (int e = threadIdx.x; e < n + k; e += blockDim.x) {
-        if (e < n) {
-            r[e] = (double)A[e * m + p];
-        } else {
-            const double c = Rrows[(e - n) * m + p];
-            ch[e - n] = (float)c;
-            cl[e - n] = (float)(c - (double)(float)c);
-        }
-    }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) r[i] = (double)A[i * m + p];
     __syncthreads();
-    __shared__ float norm2[2];  // |a_p|^2, |r|^2 after the first pass
-    auto norm_to = [&](float* out) {
-        float ss = 0.f;
-        for (int i = lane; i < n; i += 32) ss += (float)r[i] * (float)r[i];
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) *out = ss;
-    };
-    if (k > 0) {
-        if (warp == 0) norm_to(&norm2[0]);
-        subtract_projections(r, ch, cl, Q, n, k, part);
-        if (warp == 0) norm_to(&norm2[1]);
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            rh[i] = (float)r[i];
-            rl[i] = (float)(r[i] - (double)rh[i]);
-        }
-        __syncthreads();
-    }
-    // The second pass is needed where the first cancelled: a residual of at least
-    // half the column's length has lost at most one bit of orthogonality (Daniel,
-    // Gragg, Kaufman & Stewart, Math. Comp. 30 (1976)).
-    if (k > 0 && norm2[1] < 0.25f * norm2[0]) {
-        // the second pass: c_l = q_l . r, one warp per l
-        // (four at a time, their loads in flight together)
-        constexpr int NW = kPivotThreads / 32;
-        for (int l0 = warp; l0 < k; l0 += 4 * NW) {
-            float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int i = lane; i < n; i += 32) {
-                float qh[4], ql[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int l = l0 + u * NW;
-                    const float* q = Q + (long long)l * 2 * n;
-                    qh[u] = l < k ? q[i] : 0.f;
-                    ql[u] = l < k ? q[n + i] : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) ff_mul_acc(rh[i], rl[i], qh[u], ql[u], sh[u], sl[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                for (int o = 16; o > 0; o >>= 1)
-                    ff_pair_add(sh[u], sl[u], __shfl_xor_sync(0xffffffffu, sh[u], o),
-                                __shfl_xor_sync(0xffffffffu, sl[u], o));
-                if (lane == 0 && l0 + u * NW < k) {
-                    ch[l0 + u * NW] = sh[u];
-                    cl[l0 + u * NW] = sl[u];
-                }
-            }
-        }
-        __syncthreads();
-        subtract_projections(r, ch, cl, Q, n, k, part);
-    }
-    if (warp == 0) {
+    auto length2 = [&](double* out) {  // |r|^2, by one warp
         double ss = 0;
         for (int i = lane; i < n; i += 32) ss += r[i] * r[i];
         for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (lane == 0) {
-            const double nr = sqrt(ss);
-            s_inv = ss > 0 ? 1.0 / nr : 0.0;
-            rdiag[k] = nr;  // R[k][k]
+        if (lane == 0) *out = ss;
+    };
+    auto project = [&] {
+        // c_l = q_l . r, eight lanes per l (a whole warp's five double additions
+        // per l cost more than its products); r -= sum_l c_l q_l
+        constexpr int L = 8;
+        const int h = threadIdx.x % L;
+        for (int l0 = 0; l0 < k; l0 += kPivotThreads / L) {
+            const int l = l0 + threadIdx.x / L;
+            double s = 0;
+            if (l < k) {
+                const double* q = Q + (long long)l * n;
+#pragma unroll 8
+                for (int i = h; i < n; i += L) s += q[i] * r[i];
+            }
+            if (l0 + warp * (32 / L) < k)
+                for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (h == 0 && l < k) c[l] = s;
         }
+        __syncthreads();
+        subtract_projections(r, c, Q, n, k, part);
+    };
+    if (warp == kPivotThreads / 32 - 1) length2(&norm2[0]);
+    if (k > 0) {
+        project();
+        if (warp == 0) length2(&norm2[1]);
+        __syncthreads();
+        // Again where that cancelled: a residual of at least half the column's
+        // length has lost at most one bit of orthogonality (Daniel, Gragg, Kaufman
+        // & Stewart, Math. Comp. 30 (1976)).
+        if (!(norm2[1] >= 0.25 * norm2[0])) {
+            project();
+            if (warp == 0) length2(&norm2[1]);
+            __syncthreads();
+        }
+    } else {
+        if (warp == 0) length2(&norm2[1]);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double nr = sqrt(norm2[1]);
+        s_inv = norm2[1] > 0 ? 1.0 / nr : 0.0;
+        rdiag[k] = nr;  // R[k][k]
     }
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const double q = r[i] * s_inv;
         const float h = (float)q;
-        Q[(long long)k * 2 * n + i] = h;
-        Q[(long long)k * 2 * n + n + i] = (float)(q - (double)h);
+        Q[(long long)k * n + i] = q;
+        qs[i] = h;
+        qs[n + i] = (float)(q - (double)h);
     }
 }
 
 // (3): every block normalises r itself; block 0 stores q_k and |r| = R[k][k]
-// (SPLIT: q_k comes split from qr_pivot_kernel, Qs).  Double candidate columns:
+// (SPLIT: q_k comes split from qr_pivot_kernel, qs).  Double candidate columns:
 // the dots in double; single-precision ones (exact in float): in float-float
 // (ff_dot_acc).
 template <typename T, bool SPLIT>
 __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, const double* __restrict__ r, int k,
-                                 double* __restrict__ Q, const float* __restrict__ Qs, double* __restrict__ Rrows,
+                                 double* __restrict__ Q, const float* __restrict__ qs, double* __restrict__ Rrows,
                                  double* __restrict__ nu, double* __restrict__ rdiag, ArgMax* __restrict__ part) {
     extern __shared__ double q[];
     float* qh = SPLIT ? reinterpret_cast<float*>(q) : reinterpret_cast<float*>(q + n);  // float-float split of q
     float* ql = qh + n;
     if constexpr (SPLIT) {
-        for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) qh[i] = Qs[(long long)k * 2 * n + i];
+        for (int i = threadIdx.x; i < 2 * n; i += blockDim.x) qh[i] = qs[i];
         __syncthreads();
     } else {
         __shared__ double s_inv;
@@ -606,8 +567,8 @@ __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, co
     // tiles of 32 columns over one resident wave of blocks; warp g takes the
     // tile's columns (one per lane) over the row group g of 8, the groups
     // summed in shared memory
-    // (row-group sums: float pairs for single-precision columns)
-    using Part = std::conditional_t<sizeof(T) == 4, float2, double>;
+    // (row-group sums: three floats for single-precision columns)
+    using Part = std::conditional_t<sizeof(T) == 4, float3, double>;
     __shared__ Part red[8][32];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, cl = lane;
     const int rq = (n + 7) / 8, i0 = g * rq, i1 = i0 + rq < n ? i0 + rq : n;
@@ -630,8 +591,8 @@ __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, co
                     for (int u = 0; u < 8; ++u) ff_dot_acc(qh[i + u], ql[i + u], v[u], sh[u & 1], sl[u & 1]);
                 }
                 for (; i < i1; ++i) ff_dot_acc(qh[i], ql[i], (float)A[i * m + j], sh[0], sl[0]);
-                ff_pair_add(sh[0], sl[0], sh[1], sl[1]);
-                part_sum = make_float2(sh[0], sl[0]);
+                part_sum = make_float3(sh[0], sl[0], 0.f);
+                sum_pair3(part_sum.x, part_sum.y, part_sum.z, sh[1], sl[1]);
             } else {
                 double dd[4] = {0, 0, 0, 0};
                 int i = i0;
@@ -653,10 +614,11 @@ __global__ void qr_update_kernel(const T* __restrict__ A, int n, long long m, co
             if (v >= 0) {
                 double d;
                 if constexpr (sizeof(T) == 4) {
-                    float h = red[0][cl].x, lw = red[0][cl].y;
+                    float3 t = red[0][cl];
 #pragma unroll
-                    for (int gg = 1; gg < 8; ++gg) ff_pair_add(h, lw, red[gg][cl].x, red[gg][cl].y);
-                    d = (double)h + (double)lw;
+                    for (int gg = 1; gg < 8; ++gg)
+                        sum_merge3(t.x, t.y, t.z, red[gg][cl].x, red[gg][cl].y, red[gg][cl].z);
+                    d = (double)t.x + ((double)t.y + (double)t.z);
                 } else {
                     d = ((red[0][cl] + red[1][cl]) + (red[2][cl] + red[3][cl])) +
                         ((red[4][cl] + red[5][cl]) + (red[6][cl] + red[7][cl]));
@@ -826,11 +788,11 @@ cudaError_t launch_qr_step(const T* A, int n, long long m, int k, QrWork w, cuda
     const int rb = (n + 31) / 32, qb = w.blocks;
     if constexpr (sizeof(T) == 4) {
         if (n <= kPivotN) {
-            float* Qs = reinterpret_cast<float*>(w.Q);  // n x 2 x n floats in the room of n x n doubles
-            qr_pivot_kernel<<<1, kPivotThreads, 0, st>>>((const ArgMax*)w.part, qb, A, n, m, w.R, k, Qs, w.piv, w.nu,
+            float* qs = reinterpret_cast<float*>(w.r);  // [2][n] floats in the room of n doubles
+            qr_pivot_kernel<<<1, kPivotThreads, 0, st>>>((const ArgMax*)w.part, qb, A, n, m, k, w.Q, qs, w.piv, w.nu,
                                                          w.nu0, w.rdiag, w.status);
             qr_update_kernel<T, true><<<qb, kThreads, (size_t)2 * n * sizeof(float), st>>>(
-                A, n, m, nullptr, k, nullptr, Qs, w.R, w.nu, nullptr, (ArgMax*)w.part);
+                A, n, m, nullptr, k, nullptr, qs, w.R, w.nu, nullptr, (ArgMax*)w.part);
             return cudaGetLastError();
         }
     }
