@@ -35,7 +35,7 @@ template <void (*k)(PassArgs)>
 cudaError_t launch_planes(const PassArgs& a, int batch, cudaStream_t st) {
     static std::atomic<unsigned long long> done{0};
     const size_t smem = plane_smem(a.n1, a.n2);
-    cudaError_t e = kernel_limits((const void*)k, smem_max(), true, done, st);
+    cudaError_t e = kernel_limits((const void*)k, smem_max(), true, done);
     if (e != cudaSuccess) return e;
     k<<<dim3((unsigned)a.n0, (unsigned)batch), plane_threads(a.n1, a.n2), smem, st>>>(a);
     return cudaGetLastError();
@@ -46,7 +46,7 @@ cudaError_t launch_pencils(const PassArgs& a, int batch, cudaStream_t st) {
     const int units = a.n1 * a.n2 / (int)(sizeof(V) / 4);
     static std::atomic<unsigned long long> done{0};
     const size_t smem = pencil_smem(a.n0);
-    cudaError_t e = kernel_limits((const void*)pencils<V, MODE>, smem_max(), true, done, st);
+    cudaError_t e = kernel_limits((const void*)pencils<V, MODE>, smem_max(), true, done);
     if (e != cudaSuccess) return e;
     const int U = Units<V>::U;
     pencils<V, MODE><<<dim3((unsigned)((units + U - 1) / U), (unsigned)batch), 32, smem, st>>>(a, units);
@@ -59,7 +59,7 @@ cudaError_t launch_sphere(const PassArgs& a, const SphereArgs& sp, int batch, cu
     const int units = a.n1 * a.n2 / (int)(sizeof(V) / 4), U = Units<V>::U;
     const size_t smem = pencil_smem(a.n0);
     const auto k = INVERSE ? sphere_inverse<V> : sphere_forward<V>;
-    cudaError_t e = kernel_limits((const void*)k, smem_max(), true, done, st);
+    cudaError_t e = kernel_limits((const void*)k, smem_max(), true, done);
     if (e != cudaSuccess) return e;
     const int items = INVERSE ? units : sp.nlist;
     k<<<dim3((unsigned)((items + U - 1) / U), (unsigned)batch), 32, smem, st>>>(a, units, sp);

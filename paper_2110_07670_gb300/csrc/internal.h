@@ -201,8 +201,7 @@ __device__ __forceinline__ double warp_sum_ff(float v) {
 }
 #endif
 
-// True while `st` records into a CUDA graph: launchers then leave kernel
-// attributes alone (set by the same launch outside capture before).
+// True while `st` records into a CUDA graph.
 inline bool stream_capturing(cudaStream_t st) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
@@ -213,16 +212,15 @@ inline bool stream_capturing(cudaStream_t st) {
 }
 
 // Shared-memory limit (and, with full_carveout, the whole L1 carveout) of a
-// kernel, set on its first launch on each device outside stream capture: the two
-// attribute calls cost some microseconds, as much as a small launch.  `done`: a
-// static of the launcher, one bit per device.
-inline cudaError_t kernel_limits(const void* kernel, int smem, bool full_carveout, std::atomic<unsigned long long>& done,
-                                 cudaStream_t st) {
+// kernel, set before its first launch on each device, captured or not (attributes
+// are no part of a graph): the two calls cost some microseconds, as much as a small
+// launch.  `done`: a static of the launcher, one bit per device.
+inline cudaError_t kernel_limits(const void* kernel, int smem, bool full_carveout, std::atomic<unsigned long long>& done) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-    if ((done.load(std::memory_order_acquire) & bit) || stream_capturing(st)) return cudaSuccess;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess && full_carveout)
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);

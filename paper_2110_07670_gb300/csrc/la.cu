@@ -800,10 +800,10 @@ cudaError_t launch_neg_cholesky_blocked(const double* M, int n, double* L, doubl
 cudaError_t launch_neg_cholesky_inverse(const double* M, int n, double* L, double* Linv, int* status,
                                         cudaStream_t st) {
     const size_t smem = (size_t)2 * n * (n | 1) * sizeof(double);
-    static const cudaError_t attr = cudaFuncSetAttribute(neg_cholesky_inverse_kernel,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
-    if (attr != cudaSuccess) return attr;
     if (n > 64) return cudaErrorInvalidValue;
+    static std::atomic<unsigned long long> done{0};
+    cudaError_t e = kernel_limits((const void*)neg_cholesky_inverse_kernel, 72 * 1024, false, done);
+    if (e != cudaSuccess) return e;
     neg_cholesky_inverse_kernel<<<1, n <= 16 ? 128 : 512, smem, st>>>(M, n, L, Linv, status);
     return cudaGetLastError();
 }

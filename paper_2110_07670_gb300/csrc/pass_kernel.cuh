@@ -748,7 +748,7 @@ cudaError_t launch_one(const PassArgs& a, const PassShape& s, int batch, cudaStr
         if constexpr (Shape::kCube) {  // one tile size per kernel
             static std::atomic<unsigned long long> done{0};
             // three plane blocks need the whole shared carveout
-            cudaError_t e = kernel_limits((const void*)k, (int)s.smem, Shape::kMinBlocks > 2, done, st);
+            cudaError_t e = kernel_limits((const void*)k, (int)s.smem, Shape::kMinBlocks > 2, done);
             if (e != cudaSuccess) return e;
         } else if (!stream_capturing(st)) {
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);

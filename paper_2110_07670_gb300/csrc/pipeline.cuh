@@ -205,11 +205,12 @@ template <int N, int F0 = 0>
 cudaError_t pipeline_launch(const PassArgs& a, const PipeArgs& p, cudaStream_t st) {
     using G = plane_detail::Geo<N, F0>;
     auto k = pipe_detail::pair_pipeline<N, F0>;
+    static std::atomic<unsigned long long> done{0};
+    cudaError_t e = kernel_limits((const void*)k, (int)G::smem, false, done);
+    if (e != cudaSuccess) return e;
     static int per_sm = [&] {
         int b = 0;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, G::NT, G::smem) != cudaSuccess)
-            b = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, G::NT, G::smem) != cudaSuccess) b = 0;
         cudaGetLastError();
         return b;
     }();

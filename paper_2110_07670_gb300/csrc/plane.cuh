@@ -545,7 +545,7 @@ template <void (*k)(PassArgs), bool max_carveout>
 cudaError_t launch_plane(size_t smem, int n, int nt, const PassArgs& a, int batch, cudaStream_t st) {
     if (smem > 48 * 1024) {
         static std::atomic<unsigned long long> done{0};
-        cudaError_t e = kernel_limits((const void*)k, (int)smem, max_carveout, done, st);
+        cudaError_t e = kernel_limits((const void*)k, (int)smem, max_carveout, done);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)n, (unsigned)batch);

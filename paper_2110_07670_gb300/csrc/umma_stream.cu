@@ -508,8 +508,8 @@ __global__ void xi_image_kernel(const float* __restrict__ xi, int n, long long K
     *reinterpret_cast<float4*>(img + 128 * TK + o) = make_float4(l[0], l[1], l[2], l[3]);
 }
 
-cudaError_t set_smem(const void* k, std::atomic<unsigned long long>& done, cudaStream_t st) {
-    return kernel_limits(k, (int)(sizeof(WsSmem) + 1024), false, done, st);
+cudaError_t set_smem(const void* k, std::atomic<unsigned long long>& done) {
+    return kernel_limits(k, (int)(sizeof(WsSmem) + 1024), false, done);
 }
 
 }  // namespace
@@ -528,7 +528,7 @@ cudaError_t launch_gram_stream(const float* A, const float* B, int m, int n, lon
     if (K % 2 != 0 || kchunk % TK != 0 || kchunk <= 0 || ((uintptr_t)A % 8) || ((uintptr_t)B % 8))
         return cudaErrorInvalidValue;
     static std::atomic<unsigned long long> done[2];
-    cudaError_t e = set_smem(absval ? (const void*)gram_stream<true> : (const void*)gram_stream<false>, done[absval], st);
+    cudaError_t e = set_smem(absval ? (const void*)gram_stream<true> : (const void*)gram_stream<false>, done[absval]);
     if (e != cudaSuccess) return e;
     dim3 grid((m + 127) / 128, (n + 127) / 128, (unsigned)((K + kchunk - 1) / kchunk));
     if (absval)
@@ -562,7 +562,7 @@ cudaError_t launch_apply_product(int T, int n, const float* xi, long long K, con
     const int nks = (n + TK - 1) / TK;
     const void* k = Ximg ? (const void*)apply_product<true> : (const void*)apply_product<false>;
     static std::atomic<unsigned long long> done[2];
-    cudaError_t e = set_smem(k, done[Ximg != nullptr], st);
+    cudaError_t e = set_smem(k, done[Ximg != nullptr]);
     if (e != cudaSuccess) return e;
     const long long ntiles = ((K + 127) / 128) * ((T + 127) / 128);
     const unsigned grid = (unsigned)std::max<long long>(1, std::min<long long>(ntiles, sms));

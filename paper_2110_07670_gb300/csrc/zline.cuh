@@ -231,13 +231,10 @@ template <int N, int F0, bool NAT>
 cudaError_t zline_launch_nat(const PassArgs& a, int batch, cudaStream_t st) {
     constexpr int U = zline_detail::kPairsPerWarp;
     auto k = zline_detail::zline_coulomb<N, F0, NAT>;
-    static bool carveout = [&] {
-        cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaGetLastError();
-        return true;
-    }();
-    (void)carveout;
     const size_t smem = (size_t)N * U * sizeof(cx<f2>) + N * sizeof(cx<float>);
+    static std::atomic<unsigned long long> done{0};
+    cudaError_t e = kernel_limits((const void*)k, (int)smem, true, done);
+    if (e != cudaSuccess) return e;
     dim3 grid((unsigned)(((NAT ? plane_elems(N) : N * N) / 2 + U - 1) / U), (unsigned)batch);
     k<<<grid, 32, smem, st>>>(a);
     return cudaGetLastError();
