@@ -200,7 +200,7 @@ struct ace_plan {
         int status, err;
         double E;
     };
-    void* h_gamma = nullptr;  // pinned: the G = 0 coefficients of a call's vectors (gamma_begin)
+    void* h_gamma = nullptr;  // pinned: the G = 0 coefficients of a call's vectors (check_gamma_around)
     size_t hg_cap = 0;
     cudaEvent_t gamma_ev = nullptr;
     Result* h_res = nullptr;  // pinned host slots for the asynchronous build result
@@ -788,12 +788,13 @@ int check_device_error(ace_plan* P, cudaStream_t st) {
     return ACE_OK;
 }
 
-// The Gamma-point check of vectors (Im c(0) = 0) in two halves, so that the
-// copy travels behind work that touches only the plan's scratch: gamma_begin
-// enqueues the copies of one or two sets, gamma_end waits for them and judges
-// them (after a refusal, with the stream idle again).
-template <typename R>
-int gamma_begin(ace_plan* P, const void* psi, int n, const void* psi2, int n2, cudaStream_t st) {
+// The Gamma-point check of vectors (Im c(0) = 0) around work that touches only the
+// plan's scratch, so that its copy travels behind that work: the copies of one or
+// two sets are enqueued, then the work, then they are waited for and judged, also
+// where the work was refused, so that no call returns while its vectors are still
+// read.  (After a refusal at the Gamma point the stream is idle again.)
+template <typename R, class F>
+int check_gamma_around(ace_plan* P, const void* psi, int n, const void* psi2, int n2, cudaStream_t st, F&& work) {
     const size_t need = (size_t)(n + n2) * sizeof(cx<R>);
     if (need > P->hg_cap) {
         if (P->h_gamma) cudaFreeHost(P->h_gamma);
@@ -808,30 +809,29 @@ int gamma_begin(ace_plan* P, const void* psi, int n, const void* psi2, int n2, c
     if (!P->gamma_ev) ACE_CK(cudaEventCreateWithFlags(&P->gamma_ev, cudaEventDisableTiming));
     cx<R>* h = (cx<R>*)P->h_gamma;
     const size_t pitch = (size_t)P->npw * sizeof(cx<R>);
-    ACE_CK(cudaMemcpy2DAsync(h, sizeof(cx<R>), psi, pitch, sizeof(cx<R>), n, cudaMemcpyDeviceToHost, st));
-    if (n2 > 0)
-        ACE_CK(cudaMemcpy2DAsync(h + n, sizeof(cx<R>), psi2, pitch, sizeof(cx<R>), n2, cudaMemcpyDeviceToHost, st));
-    ACE_CK(cudaEventRecord(P->gamma_ev, st));
-    return ACE_OK;
-}
-
-template <typename R>
-int gamma_end(ace_plan* P, int n, int n2, cudaStream_t st) {
+    cudaError_t e = cudaMemcpy2DAsync(h, sizeof(cx<R>), psi, pitch, sizeof(cx<R>), n, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && n2 > 0)
+        e = cudaMemcpy2DAsync(h + n, sizeof(cx<R>), psi2, pitch, sizeof(cx<R>), n2, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaEventRecord(P->gamma_ev, st);
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(st);
+        cudaGetLastError();
+        return fail(ACE_ERR_CUDA, std::string("Gamma-point check: ") + cudaGetErrorString(e));
+    }
+    const int rc = work();
     ACE_CK(cudaEventSynchronize(P->gamma_ev));
-    const cx<R>* h = (const cx<R>*)P->h_gamma;
     for (int i = 0; i < n + n2; ++i)
         if (std::fabs((double)h[i].im) > 1e-6) {
             ACE_CK(cudaStreamSynchronize(st));
             return fail(ACE_ERR_INVALID_ARG,
                         "Im c(G=0) of vector " + std::to_string(i < n ? i : i - n) + " is not zero");
         }
-    return ACE_OK;
+    return rc;
 }
 
 template <typename R>
 int check_gamma(ace_plan* P, const void* psi, int n, cudaStream_t st) {
-    ACE_TRY(gamma_begin<R>(P, psi, n, nullptr, 0, st));
-    return gamma_end<R>(P, n, 0, st);
+    return check_gamma_around<R>(P, psi, n, nullptr, 0, st, [] { return ACE_OK; });
 }
 
 // The quads go through the plan's pinned staging buffer (a captured copy
@@ -880,43 +880,44 @@ int upload_quads(ace_plan* P, const std::vector<Quad>& q, cudaStream_t st) {
 template <typename R>
 int pairs_enqueue(ace_plan* P, const void* psi_G, int n_occ, double alpha, const int32_t* rp, const int32_t* col,
                   void* WG_out, cudaStream_t st, bool check) {
-    if (check) ACE_TRY(gamma_begin<R>(P, psi_G, n_occ, nullptr, 0, st));
-    std::vector<int> pa, pb;
-    if (rp) {
-        if (rp[0] != 0) return fail(ACE_ERR_INVALID_ARG, "pair_row_ptr[0] must be 0");
-        for (int i = 0; i < n_occ; ++i) {
-            if (rp[i + 1] < rp[i]) return fail(ACE_ERR_INVALID_ARG, "pair_row_ptr not monotone");
-            for (int t = rp[i]; t < rp[i + 1]; ++t) {
-                if (col[t] < i || col[t] >= n_occ) return fail(ACE_ERR_INVALID_ARG, "pair column out of range");
-                pa.push_back(i);
-                pb.push_back(col[t]);
-            }
-        }
-    } else {
-        for (int i = 0; i < n_occ; ++i)
-            for (int j = i; j < n_occ; ++j) {
-                pa.push_back(i);
-                pb.push_back(j);
-            }
-    }
-    std::vector<Quad> oq = orbital_quads(n_occ), q = oq;
+    const std::vector<Quad> oq = orbital_quads(n_occ);
     const int n_orb_t = (int)oq.size();
-    if (P->pair_tile > 0) {
-        tile_pairs(pa, pb, P->pair_tile);
-        pack_pairs(pa, pb, q);
-    } else {
-        pack_pairs_blocked(n_occ, pa, pb, P->row_block, q);
-    }
-    const int n_pair_t = (int)q.size() - n_orb_t;
-    ACE_TRY(upload_quads(P, q, st));
-    const Quad* d_oq = P->d_quads;
-    const Quad* d_pq = P->d_quads + n_orb_t;
-
-    const cx<R>* psi = (const cx<R>*)psi_G;
+    int n_pair_t = 0;
     R* phi = (R*)P->d_phi;
     R* acc = (R*)P->d_acc;
-    ACE_TRY(run_to_real<R>(P, psi, d_oq, n_orb_t, phi, st));
-    if (check) ACE_TRY(gamma_end<R>(P, n_occ, 0, st));
+    auto orbitals = [&]() -> int {
+        std::vector<int> pa, pb;
+        if (rp) {
+            if (rp[0] != 0) return fail(ACE_ERR_INVALID_ARG, "pair_row_ptr[0] must be 0");
+            for (int i = 0; i < n_occ; ++i) {
+                if (rp[i + 1] < rp[i]) return fail(ACE_ERR_INVALID_ARG, "pair_row_ptr not monotone");
+                for (int t = rp[i]; t < rp[i + 1]; ++t) {
+                    if (col[t] < i || col[t] >= n_occ) return fail(ACE_ERR_INVALID_ARG, "pair column out of range");
+                    pa.push_back(i);
+                    pb.push_back(col[t]);
+                }
+            }
+        } else {
+            for (int i = 0; i < n_occ; ++i)
+                for (int j = i; j < n_occ; ++j) {
+                    pa.push_back(i);
+                    pb.push_back(j);
+                }
+        }
+        std::vector<Quad> q = oq;
+        if (P->pair_tile > 0) {
+            tile_pairs(pa, pb, P->pair_tile);
+            pack_pairs(pa, pb, q);
+        } else {
+            pack_pairs_blocked(n_occ, pa, pb, P->row_block, q);
+        }
+        n_pair_t = (int)q.size() - n_orb_t;
+        ACE_TRY(upload_quads(P, q, st));
+        return run_to_real<R>(P, (const cx<R>*)psi_G, P->d_quads, n_orb_t, phi, st);
+    };
+    ACE_TRY(check ? check_gamma_around<R>(P, psi_G, n_occ, nullptr, 0, st, orbitals) : orbitals());
+    const Quad* d_oq = P->d_quads;
+    const Quad* d_pq = P->d_quads + n_orb_t;
     ACE_CK(cudaMemsetAsync(acc, 0, (size_t)n_occ * P->N * sizeof(R), st));
     ACE_TRY(grow(&P->d_epart, &P->epart_cap, (size_t)std::max(n_pair_t, 1) * P->ntiles_last * 2));
     ACE_TRY(run_pairs<R>(P, phi, phi, acc, acc, 1, d_pq, n_pair_t, P->d_epart, st));
@@ -1003,36 +1004,36 @@ int build_impl(ace_plan* P, const void* psi_G, int n_occ, double alpha, const in
 template <typename R>
 int hfx_impl(ace_plan* P, const void* psi_occ, int n_occ, double alpha, const void* psi, int T, void* out,
              cudaStream_t st) {
-    ACE_TRY(gamma_begin<R>(P, psi_occ, n_occ, psi, T, st));
-    std::vector<Quad> oq = orbital_quads(n_occ), tq = orbital_quads(T), q = oq;
-    q.insert(q.end(), tq.begin(), tq.end());
-    std::vector<int> pa, pb;
-    for (int t = 0; t < T; ++t)
-        for (int j = 0; j < n_occ; ++j) {
-            pa.push_back(t);
-            pb.push_back(j);
-        }
-    pack_pairs(pa, pb, q);
-    const int no = (int)oq.size(), nt = (int)tq.size(), np = (int)q.size() - no - nt;
-    ACE_TRY(upload_quads_eager(P, q, st));
-    size_t tcap_elems = P->t_cap;
-    void* tphi = P->d_tphi;
-    if ((size_t)T * P->N > tcap_elems) {
-        if (P->d_tphi) cudaFree(P->d_tphi);
-        if (P->d_tacc) cudaFree(P->d_tacc);
-        P->d_tphi = P->d_tacc = nullptr;
-        P->t_cap = 0;
-        ACE_TRY(dalloc(&P->d_tphi, (size_t)T * P->N * sizeof(R)));
-        ACE_TRY(dalloc(&P->d_tacc, (size_t)T * P->N * sizeof(R)));
-        P->t_cap = (size_t)T * P->N;
-        tphi = P->d_tphi;
-    }
+    const std::vector<Quad> oq = orbital_quads(n_occ), tq = orbital_quads(T);
+    const int no = (int)oq.size(), nt = (int)tq.size();
+    int np = 0;
     R* phi = (R*)P->d_phi;
-    ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi_occ, P->d_quads, no, phi, st));
-    ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi, P->d_quads + no, nt, (R*)tphi, st));
-    ACE_TRY(gamma_end<R>(P, n_occ, T, st));
+    ACE_TRY(check_gamma_around<R>(P, psi_occ, n_occ, psi, T, st, [&]() -> int {
+        std::vector<Quad> q = oq;
+        q.insert(q.end(), tq.begin(), tq.end());
+        std::vector<int> pa, pb;
+        for (int t = 0; t < T; ++t)
+            for (int j = 0; j < n_occ; ++j) {
+                pa.push_back(t);
+                pb.push_back(j);
+            }
+        pack_pairs(pa, pb, q);
+        np = (int)q.size() - no - nt;
+        ACE_TRY(upload_quads_eager(P, q, st));
+        if ((size_t)T * P->N > P->t_cap) {
+            if (P->d_tphi) cudaFree(P->d_tphi);
+            if (P->d_tacc) cudaFree(P->d_tacc);
+            P->d_tphi = P->d_tacc = nullptr;
+            P->t_cap = 0;
+            ACE_TRY(dalloc(&P->d_tphi, (size_t)T * P->N * sizeof(R)));
+            ACE_TRY(dalloc(&P->d_tacc, (size_t)T * P->N * sizeof(R)));
+            P->t_cap = (size_t)T * P->N;
+        }
+        ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi_occ, P->d_quads, no, phi, st));
+        return run_to_real<R>(P, (const cx<R>*)psi, P->d_quads + no, nt, (R*)P->d_tphi, st);
+    }));
     ACE_CK(cudaMemsetAsync(P->d_tacc, 0, (size_t)T * P->N * sizeof(R), st));
-    ACE_TRY(run_pairs<R>(P, (const R*)tphi, phi, (R*)P->d_tacc, nullptr, 0, P->d_quads + no + nt, np, nullptr, st));
+    ACE_TRY(run_pairs<R>(P, (const R*)P->d_tphi, phi, (R*)P->d_tacc, nullptr, 0, P->d_quads + no + nt, np, nullptr, st));
     const double g = phi_gain<R>(P);
     ACE_TRY(run_to_recip<R>(P, (const R*)P->d_tacc, P->d_quads + no, nt,
                             -alpha * std::sqrt(P->omega) / (double)P->N / (g * g * g), (cx<R>*)out, st));
@@ -1048,13 +1049,13 @@ int hfx_impl(ace_plan* P, const void* psi_occ, int n_occ, double alpha, const vo
 template <typename R>
 int overlap_impl(ace_plan* P, const void* psi_G, int n, double rho_cut, int32_t* rp, int32_t* col, int* n_pairs,
                  double* S_out, cudaStream_t st) {
-    ACE_TRY(gamma_begin<R>(P, psi_G, n, nullptr, 0, st));
-    std::vector<Quad> oq = orbital_quads(n);
-    ACE_TRY(upload_quads_eager(P, oq, st));
-    ACE_TRY(grow(&P->d_S, &P->S_cap, (size_t)n * n));
+    const std::vector<Quad> oq = orbital_quads(n);
     R* phi = (R*)P->d_phi;
-    ACE_TRY(run_to_real<R>(P, (const cx<R>*)psi_G, P->d_quads, (int)oq.size(), phi, st));
-    ACE_TRY(gamma_end<R>(P, n, 0, st));
+    ACE_TRY(check_gamma_around<R>(P, psi_G, n, nullptr, 0, st, [&]() -> int {
+        ACE_TRY(upload_quads_eager(P, oq, st));
+        ACE_TRY(grow(&P->d_S, &P->S_cap, (size_t)n * n));
+        return run_to_real<R>(P, (const cx<R>*)psi_G, P->d_quads, (int)oq.size(), phi, st);
+    }));
     const long long K = P->N;
     const double g = phi_gain<R>(P);
     const double scale = P->omega / (double)P->N / (g * g);
@@ -1272,8 +1273,9 @@ int apply_energy_impl(ace_plan* P, const void* xi, int n_occ, const void* psi, i
 }
 
 void free_plan(ace_plan* P) {
-    if (P->gamma_ev) cudaEventDestroy(P->gamma_ev);
+    if (P->gamma_ev) cudaEventSynchronize(P->gamma_ev);
     if (P->h_gamma) cudaFreeHost(P->h_gamma);
+    if (P->gamma_ev) cudaEventDestroy(P->gamma_ev);
     if (P->h_res) cudaFreeHost(P->h_res);
     if (P->quads_ev) cudaEventSynchronize(P->quads_ev);
     if (P->h_quads) cudaFreeHost(P->h_quads);
