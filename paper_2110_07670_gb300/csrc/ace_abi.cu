@@ -344,7 +344,8 @@ int setup_shapes(ace_plan* P) {
         P->s_z = mk_shape(n0, ty, tx, 4);
     }
     // single precision: the runtime-size kernels take every box they can hold
-    // (measured against the tile passes: see generic.cuh)
+    // (measured against the tile passes: see generic.cuh); planes and pencils
+    // beyond a block's shared memory and extents of one stay with the tile passes
     if (sizeof(R) == 4 && generic_supported(n0, n1, n2)) {
         P->gen = P->fused_xy = true;
         P->s_xy = mk_shape(1, n1, n2, 3);
