@@ -1256,8 +1256,10 @@ int apply_energy_impl(ace_plan* P, const void* xi, int n_occ, const void* psi, i
             int nchunk;
             mark(P, PH_GRAM, st);
             ACE_TRY(gram_partials(P, (const float*)psi, T, (const float*)xi, n_occ, &part, &nchunk, st));
+            mark(P, PH_ENERGY, st);
             ACE_CKL(launch_gram_finish_sumsq(part, nchunk, (const float*)psi, (const float*)xi, T, n_occ, 2LL * P->npw,
                                              P->d_C, -1.0, P->d_E, st));
+            ++P->launches;  // two kernels
             done = true;
         }
     }
