@@ -132,9 +132,10 @@ int ace_plan_config(const ace_plan* plan, int* pair_variant, int* pair_streams, 
  * creation times the four at the chosen pair_variant (row_block_ms[4], 0 =
  * not timed) unless the environment fixes ACE_ROW_BLOCK.  With ACE_TUNE_CACHE
  * naming a file, the choice of pair_variant, pair_streams and row_block is
- * looked up there by grid, n_occ_max, precision and device before any timing
- * and appended after it (*from_cache = 1 when it came from the file).  Any
- * output may be NULL. */
+ * looked up there by grid, n_occ_max, precision, device and the revision of the
+ * kernels (lines of other revisions do not count) before any timing and
+ * appended after it (*from_cache = 1 when it came from the file).  Any output
+ * may be NULL. */
 int ace_plan_tuning(const ace_plan* plan, int* row_block, float* row_block_ms, int* from_cache);
 
 /* The radix plan of the pair passes' 3D FFTs (the Poisson solves of Eq. 3):

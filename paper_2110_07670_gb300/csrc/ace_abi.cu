@@ -1318,6 +1318,10 @@ int pair_tables(ace_plan* P, int r0);
 // First radix of the pair passes' plan: r0, or make_axis_plan's for r0 = 0.
 int first_radix(const ace_plan* P, int r0) { return r0 ? r0 : (P->ax[0].nstages > 0 ? P->ax[0].radix[0] : 1); }
 
+// Revision of the pair kernels in the tune cache's lines, raised when a variant
+// changes its kernels or its speed: a choice timed on others does not count.
+constexpr int kPairKernels = 2;
+
 template <typename R>
 int choose_pair_variant(ace_plan* P, const ace_opts* opts) {
     const int req = opts ? opts->pair_variant : 0;
@@ -1373,7 +1377,8 @@ int choose_pair_variant(ace_plan* P, const ace_opts* opts) {
         set_variant(P, 1, fixed_streams ? fixed_streams : 2);
         return ACE_OK;
     }
-    // the tune cache: one line per (grid, n_occ_max, precision, device)
+    // the tune cache: one line per (grid, n_occ_max, precision, device, revision
+    // of the kernels that were timed)
     char key[256] = {0};
     const char* cache = std::getenv("ACE_TUNE_CACHE");
     if (cache && *cache && !fixed_streams) {
@@ -1384,8 +1389,8 @@ int choose_pair_variant(ace_plan* P, const ace_opts* opts) {
         }
         for (char* c = prop.name; *c; ++c)
             if (*c == ' ') *c = '_';
-        std::snprintf(key, sizeof key, "%dx%dx%d n%d f%d %s sm%d", P->n[0], P->n[1], P->n[2], P->n_occ_max,
-                      (int)sizeof(R) * 8, prop.name, P->sms);
+        std::snprintf(key, sizeof key, "%dx%dx%d n%d f%d %s sm%d k%d", P->n[0], P->n[1], P->n[2], P->n_occ_max,
+                      (int)sizeof(R) * 8, prop.name, P->sms, kPairKernels);
         if (FILE* f = std::fopen(cache, "r")) {
             char line[512];
             int v = 0, st = 0, rb = -1, r0 = 0;
