@@ -1,7 +1,8 @@
 """SCDM's pivot and column kernels at the edges of their sizes: one and a few
 orbitals, rows that are and are not a multiple of a warp, the largest set of the
-one-block pivot kernel and one beyond it, nearly dependent orbitals (the second
-Gram-Schmidt pass runs), both precisions where the kernels differ."""
+one-block pivot kernel (160) and one beyond it, sets well beyond, nearly dependent
+orbitals (the second Gram-Schmidt pass runs), both precisions where the kernels
+differ."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,prec", [(1, "mixed"), (2, "mixed"), (31, "mixed"), (33, "mixed"), (100, "mixed"),
-                                    (256, "mixed"), (257, "mixed"), (33, "fp64")])
+                                    (160, "mixed"), (161, "mixed"), (256, "mixed"), (257, "mixed"),
+                                    (33, "fp64")])
 def test_scdm_sizes_match_oracle(n, prec):
     cell, ecut = gen.cubic_cell(8.0), 25.0
     psi = gen.random_orbitals(cell, ecut, n, seed=600 + n)
